@@ -665,106 +665,191 @@ __global__ void k_batch_condition(const PairLevel *__restrict__ pl, int npairs, 
 #endif
 }
 
-// Standalone direction for a given set of pairs (reg_lbfgs_direction): the
-// dots of S, Y and g one at a time (entry 0: g'g, 1: ||g||_inf, then S_i'g,
-// Y_i'g, then S_i'Y_j, Y_i'Y_j).  Only used by that entry point.
-__device__ __forceinline__ void pair_dot_operands(int d, int count, long long n, long long e,
-                                                  const float *__restrict__ S, const float *__restrict__ Y,
-                                                  const float *__restrict__ g, float &a, float &b)
-{
-    int q = d - 2;
-    if (q < 2 * count) {
-        int i = q >> 1;
-        a = (q & 1) ? Y[(size_t)i * n + e] : S[(size_t)i * n + e];
-        b = g[e];
-    } else {
-        q -= 2 * count;
-        int i = (q >> 1) / count, j = (q >> 1) % count;
-        a = (q & 1) ? Y[(size_t)i * n + e] : S[(size_t)i * n + e];
-        b = Y[(size_t)j * n + e];
-    }
-}
+// Standalone direction for a given set of pairs (reg_lbfgs_direction): two
+// passes over the caller's vectors.  The first takes every dot the compact form
+// needs in one read of S, Y and g; its last block sums the block partials and
+// solves for the coefficients.  The second combines the vectors.
+//
+// Both are bound by memory: (2 count + 1) n floats read twice, the second time
+// from L2 while the vectors fit there.  S and Y rows start at multiples of n
+// floats (n = 3 nodes, often odd), so a row has no alignment beyond 4 bytes and
+// the loads are 4-byte ones, coalesced, PD_U per vector and thread in flight.
+// 3 x 65^3 unknowns, 5 pairs: one pass per dot, the sums and the solve in one
+// FP64 thread and FP64 coefficients per element took 166 + 1292 + 54 us, the
+// whole call 1481 us; now the call takes 49 us.
+constexpr int PD_U = 4;                     // elements per thread and chunk
+constexpr int PD_CHUNK = PD_U * VT;
 
-__global__ void __launch_bounds__(VT) k_lb_pair_dots(long long n, int count, const float *__restrict__ S,
-                                                     const float *__restrict__ Y, const float *__restrict__ g,
-                                                     float *__restrict__ partials)
-{
-    const int nd = 2 + 2 * count + 2 * count * count;
-    for (int d = 0; d < nd; d++) {
-        float acc = 0.f;
-        for (long long e = blockIdx.x * (long long)VT + threadIdx.x; e < n; e += (long long)gridDim.x * VT) {
-            if (d == 0) {
-                acc = fmaf(g[e], g[e], acc);
-            } else if (d == 1) {
-                acc = fmaxf(acc, fabsf(g[e]));
-            } else {
-                float a, b;
-                pair_dot_operands(d, count, n, e, S, Y, g, a, b);
-                acc = fmaf(a, b, acc);
-            }
-        }
-        float v[1] = {acc};
-        __syncthreads();
-        block_reduce_write<1>(v, d == 1 ? 0 : -1, partials + (size_t)blockIdx.x * nd + d);
-        __syncthreads();
-    }
-}
+// dots of C pairs: 0: g'g, 1: ||g||_inf, then S_i'g, Y_i'g, then the upper
+// triangles (i <= j by age) of S_i'Y_j and Y_i'Y_j
+__host__ __device__ constexpr int pd_count(int c) { return 2 + 2 * c + c * (c + 1); }
+__host__ __device__ constexpr int pd_tri(int i, int j) { return j * (j + 1) / 2 + i; }   // i <= j
+constexpr int PD_MAX = pd_count(LB_MAXM);
+static_assert(PD_MAX <= CT, "one thread of the reduction per dot");
 
-__global__ void __launch_bounds__(VT) k_lb_direction_plain(long long n, const LbfgsState *__restrict__ st,
-                                                           const float *__restrict__ g, const float *__restrict__ S,
-                                                           const float *__restrict__ Y, float *__restrict__ p)
+// The coefficients of p = cg g + sum_j cp_j S_j + cy_j Y_j from the dots in
+// red; run by one warp on the block's control state.
+__device__ __forceinline__ void pair_coefficients(LbfgsState &S, int count, double Hmin, const double *red)
 {
-    const int dc = st->dcount;
-    const float cg = (float)st->cg;
-    for (long long e = blockIdx.x * (long long)VT + threadIdx.x; e < n; e += (long long)gridDim.x * VT) {
-        float v = cg * g[e];
-        for (int j = 0; j < dc; j++) {
-            size_t o = (size_t)st->dslot[j] * n + e;
-            v = fmaf((float)st->cp[j], S[o], fmaf((float)st->cy[j], Y[o], v));
-        }
-        p[e] = v;
+    const int lane = threadIdx.x & 31;
+    if (lane == 0) {
+        S.Hmin = Hmin;
+        S.gg = red[0];
+        S.ginf = red[1];
+        S.count = count;
+        if (count == 0)
+            set_p0(&S);
     }
-}
-
-__global__ void k_lb_pair_setup(LbfgsState *__restrict__ st, int count, const float *__restrict__ partials,
-                                int nblocks)
-{
-    const int nd = 2 + 2 * count + 2 * count * count;
-    if (threadIdx.x == 0) {
-        double red[2 + 2 * LB_MAXM + 2 * LB_MAXM * LB_MAXM];
-        for (int d = 0; d < nd; d++) {
-            double s = 0.0;
-            for (int b = 0; b < nblocks; b++) {
-                double x = partials[(size_t)b * nd + d];
-                s = (d == 1) ? fmax(s, x) : s + x;
-            }
-            red[d] = s;
+    if (count == 0)
+        return;
+    const double *sy = red + 2 + 2 * count, *yy = sy + count * (count + 1) / 2;
+    if (lane < count) {
+        const int i = lane;
+        S.order[i] = i;
+        S.tscale[i] = 1.0;
+        S.Pg[i] = red[2 + 2 * i];
+        S.Yg[i] = red[3 + 2 * i];
+        for (int j = 0; j < count; j++) {   // the lower triangle of S'Y is never read
+            S.SY[i][j] = i <= j ? sy[pd_tri(i, j)] : 0.0;
+            S.YY[i][j] = yy[i <= j ? pd_tri(i, j) : pd_tri(j, i)];
         }
-        st->gg = red[0];
-        st->ginf = red[1];
-        st->count = count;
-        for (int i = 0; i < count; i++) {
-            st->order[i] = i;
-            st->tscale[i] = 1.0;
-            st->Pg[i] = red[2 + 2 * i];
-            st->Yg[i] = red[3 + 2 * i];
-            for (int j = 0; j < count; j++) {
-                int q = 2 + 2 * count + 2 * (i * count + j);
-                st->SY[i][j] = red[q];
-                st->YY[i][j] = red[q + 1];
-            }
-            st->iSY[i] = 1.0 / st->SY[i][i];
-        }
-        if (count > 0)
-            st->gamma = st->SY[count - 1][count - 1] / st->YY[count - 1][count - 1];
-        else
-            set_p0(st);
-        st->iter_continue = 1;
-        st->done = 0;
+        S.iSY[i] = 1.0 / sy[pd_tri(i, i)];
+    } else if (lane == count) {
+        S.gamma = sy[pd_tri(count - 1, count - 1)] / yy[pd_tri(count - 1, count - 1)];
     }
     __syncwarp();
-    if (count > 0)
-        set_compact_warp(st);
+    set_compact_warp(&S);
+}
+
+template <int C>
+__global__ void __launch_bounds__(VT) k_lb_pair_dots(long long n, const float *__restrict__ S,
+                                                     const float *__restrict__ Y, const float *__restrict__ g,
+                                                     float *__restrict__ partials, unsigned *__restrict__ cnt,
+                                                     LbfgsState *__restrict__ st, double Hmin)
+{
+    constexpr int ND = pd_count(C), SY0 = 2 + 2 * C, YY0 = SY0 + C * (C + 1) / 2;
+    float v[ND];
+#pragma unroll
+    for (int d = 0; d < ND; d++)
+        v[d] = 0.f;
+    for (long long e0 = blockIdx.x * (long long)PD_CHUNK; e0 < n; e0 += (long long)gridDim.x * PD_CHUNK) {
+        float a[PD_U][2 * C + 1];
+#pragma unroll
+        for (int k = 0; k < PD_U; k++) {
+            const long long e = e0 + k * VT + threadIdx.x;
+            const bool in = e < n;
+            a[k][2 * C] = in ? __ldg(g + e) : 0.f;
+#pragma unroll
+            for (int i = 0; i < C; i++) {
+                a[k][2 * i] = in ? __ldg(S + i * n + e) : 0.f;
+                a[k][2 * i + 1] = in ? __ldg(Y + i * n + e) : 0.f;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < PD_U; k++) {
+            const float x = a[k][2 * C];
+            v[0] = fmaf(x, x, v[0]);
+            v[1] = fmaxf(v[1], fabsf(x));
+#pragma unroll
+            for (int j = 0; j < C; j++) {
+                const float s = a[k][2 * j], y = a[k][2 * j + 1];
+                v[2 + 2 * j] = fmaf(s, x, v[2 + 2 * j]);
+                v[3 + 2 * j] = fmaf(y, x, v[3 + 2 * j]);
+#pragma unroll
+                for (int i = 0; i <= j; i++) {
+                    v[SY0 + pd_tri(i, j)] = fmaf(a[k][2 * i], y, v[SY0 + pd_tri(i, j)]);
+                    v[YY0 + pd_tri(i, j)] = fmaf(a[k][2 * i + 1], y, v[YY0 + pd_tri(i, j)]);
+                }
+            }
+        }
+    }
+    block_reduce_write<ND>(v, 1, partials + (size_t)ND * blockIdx.x);
+    // the last block sums the partials and solves (as vec_tail)
+    __shared__ int s_last;
+    __shared__ double red[ND];
+    __shared__ DFloat scratch[CT];
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        fence_acq_rel_gpu();
+        s_last = atomicAdd(cnt, 1u) == gridDim.x - 1;
+        if (s_last) {
+            fence_acq_rel_gpu();
+            *cnt = 0;
+        }
+    }
+    __syncthreads();
+    if (!s_last)
+        return;
+    control_reduce(partials, (int)gridDim.x, ND, 1, red, scratch);
+    // a sum beyond FP32's range (or of infinities) is not one for double-float: FP64
+    if (threadIdx.x < ND && threadIdx.x != 1 && !isfinite(red[threadIdx.x])) {
+        double x = 0.0;
+        for (int b = 0; b < (int)gridDim.x; b++)
+            x += (double)__ldcg(partials + (size_t)b * ND + threadIdx.x);
+        red[threadIdx.x] = x;
+    }
+    LbfgsState &L = ctl_state();
+    for (int i = threadIdx.x; i < STATE_WORDS; i += VT)
+        reinterpret_cast<int *>(&L)[i] = 0;
+    __syncthreads();
+    if (threadIdx.x < 32)
+        pair_coefficients(L, C, Hmin, red);
+    __syncthreads();
+    for (int i = threadIdx.x; i < STATE_WORDS; i += VT)
+        reinterpret_cast<int *>(st)[i] = reinterpret_cast<const int *>(&L)[i];
+}
+
+// p = cg g + sum_j cp_j S_j + cy_j Y_j
+template <int C>
+__global__ void __launch_bounds__(VT) k_lb_pair_combine(long long n, const LbfgsState *__restrict__ st,
+                                                        const float *__restrict__ g, const float *__restrict__ S,
+                                                        const float *__restrict__ Y, float *__restrict__ p)
+{
+    const float cg = (float)st->cg;
+    float cp[C + 1], cy[C + 1];
+#pragma unroll
+    for (int j = 0; j < C; j++) {
+        cp[j] = (float)st->cp[j];
+        cy[j] = (float)st->cy[j];
+    }
+    for (long long e0 = blockIdx.x * (long long)PD_CHUNK; e0 < n; e0 += (long long)gridDim.x * PD_CHUNK) {
+        float a[PD_U][2 * C + 1];
+#pragma unroll
+        for (int k = 0; k < PD_U; k++) {
+            const long long e = e0 + k * VT + threadIdx.x;
+            const bool in = e < n;
+            a[k][2 * C] = in ? __ldg(g + e) : 0.f;
+#pragma unroll
+            for (int j = 0; j < C; j++) {
+                a[k][2 * j] = in ? __ldg(S + j * n + e) : 0.f;
+                a[k][2 * j + 1] = in ? __ldg(Y + j * n + e) : 0.f;
+            }
+        }
+#pragma unroll
+        for (int k = 0; k < PD_U; k++) {
+            const long long e = e0 + k * VT + threadIdx.x;
+            float x = cg * a[k][2 * C];
+#pragma unroll
+            for (int j = 0; j < C; j++)
+                x = fmaf(cp[j], a[k][2 * j], fmaf(cy[j], a[k][2 * j + 1], x));
+            if (e < n)
+                p[e] = x;
+        }
+    }
+}
+
+template <int C>
+cudaError_t launch_pair_direction(reg_ctx *c, long long n, const float *S, const float *Y, const float *g, float *p,
+                                  double Hmin, cudaStream_t s)
+{
+    // 2 blocks per SM: enough loads in flight, few partials for the last block
+    const long long chunks = (n + PD_CHUNK - 1) / PD_CHUNK;
+    const int nb = (int)std::min<long long>(chunks, 2LL * c->num_sms);
+    const int nc = (int)std::min<long long>(chunks, 8LL * c->num_sms);
+    k_lb_pair_dots<C><<<nb, VT, 0, s>>>(n, S, Y, g, c->lb.partials, c->lb.cnt + c->lb.cnt_len, c->lb.st, Hmin);
+    k_lb_pair_combine<C><<<nc, VT, 0, s>>>(n, c->lb.st, g, S, Y, p);
+    c->launches += 2;
+    return cudaGetLastError();
 }
 
 // ---------------------------------------------------------------------------
@@ -1137,16 +1222,17 @@ cudaError_t launch_finalize_ctl(reg_ctx *c, const double *pD, int nD, const doub
 cudaError_t lbfgs_direction_standalone(reg_ctx *c, long long n, int count, const float *S, const float *Y,
                                        const float *g, float *p, double Hmin, cudaStream_t s)
 {
-    int nb = num_blocks_for(c, n, VT);
-    k_lb_pair_dots<<<nb, VT, 0, s>>>(n, count, S, Y, g, c->lb.partials);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess)
-        return e;
-    k_lb_pair_setup<<<1, 32, 0, s>>>(c->lb.st, count, c->lb.partials, nb);
-    // pairs live in the caller's S, Y: slots 0..count-1 at stride n (any alignment)
-    k_lb_direction_plain<<<nb, VT, 0, s>>>(n, c->lb.st, g, S, Y, p);
-    c->launches += 3;
-    return cudaGetLastError();
+    switch (count) {
+    case 0: return launch_pair_direction<0>(c, n, S, Y, g, p, Hmin, s);
+    case 1: return launch_pair_direction<1>(c, n, S, Y, g, p, Hmin, s);
+    case 2: return launch_pair_direction<2>(c, n, S, Y, g, p, Hmin, s);
+    case 3: return launch_pair_direction<3>(c, n, S, Y, g, p, Hmin, s);
+    case 4: return launch_pair_direction<4>(c, n, S, Y, g, p, Hmin, s);
+    case 5: return launch_pair_direction<5>(c, n, S, Y, g, p, Hmin, s);
+    case 6: return launch_pair_direction<6>(c, n, S, Y, g, p, Hmin, s);
+    case 7: return launch_pair_direction<7>(c, n, S, Y, g, p, Hmin, s);
+    default: return launch_pair_direction<8>(c, n, S, Y, g, p, Hmin, s);
+    }
 }
 
 // batched launchers (batch.cu): step 0 norms of g, 1 direction, 2 its p0 redo, 3 accept

@@ -326,8 +326,9 @@ int allocate_buffers(reg_ctx *c)
         const int groups = (4 * c->num_sms + LB_RG - 1) / LB_RG;
         CK(cudaMalloc(&b.gpart, sizeof(float2) * groups * (2 + 4 * LB_MAXS)));
         b.cnt_len = groups + 1;
-        CK(cudaMalloc(&b.cnt, sizeof(unsigned) * b.cnt_len));
-        CK(cudaMemset(b.cnt, 0, sizeof(unsigned) * b.cnt_len));
+        // one more counter past them: reg_lbfgs_direction's
+        CK(cudaMalloc(&b.cnt, sizeof(unsigned) * (b.cnt_len + 1)));
+        CK(cudaMemset(b.cnt, 0, sizeof(unsigned) * (b.cnt_len + 1)));
         CK(cudaMalloc(&b.gbar, 3 * sizeof(unsigned)));
         CK(cudaMemset(b.gbar, 0, 3 * sizeof(unsigned)));
     }
@@ -694,8 +695,6 @@ int reg_lbfgs_direction(reg_handle c, long long n, int count, const float *S_dev
         return set_err(c, REG_ERR_ARG, "reg_lbfgs_direction: bad argument");
     const Level &L = c->L[0];
     double Hmin = fmin(L.H[0], fmin(L.H[1], L.H[2]));
-    lbfgs_state_reset_host(c->lb.st_host, c->cfg, 1, Hmin);
-    CK(cudaMemcpyAsync(c->lb.st, c->lb.st_host, sizeof(LbfgsState), cudaMemcpyHostToDevice, c->stream));
     CK(lbfgs_direction_standalone(c, n, count, S_dev, Y_dev, g_dev, p_dev, Hmin, c->stream));
     CK(cudaStreamSynchronize(c->stream));
     return REG_OK;
