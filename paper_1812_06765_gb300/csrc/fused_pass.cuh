@@ -329,6 +329,77 @@ __device__ __forceinline__ float ldimg_zero_ext(const IMG *T, int mx, int my, in
     return in ? ldimg(T + (x + mx * (y + my * z))) : 0.f;
 }
 
+// Trilinear interpolation of both columns' samples from their corners
+// (0 = (0,0,0), 1 = (1,0,0), 2 = (0,1,0), 3 = (1,1,0), 4..7 the same at z + 1)
+// and fractions: the value and the interpolant's differences per voxel.
+__device__ __forceinline__ void interp_pair(const float2 pc[8], const float2 fr[3], float2 &val, float2 &gx, float2 &gy,
+                                            float2 &gz)
+{
+    const float2 d00 = sub2(pc[1], pc[0]), d10 = sub2(pc[3], pc[2]);
+    const float2 d01 = sub2(pc[5], pc[4]), d11 = sub2(pc[7], pc[6]);
+    const float2 a00 = fma2(fr[0], d00, pc[0]), a10 = fma2(fr[0], d10, pc[2]);
+    const float2 a01 = fma2(fr[0], d01, pc[4]), a11 = fma2(fr[0], d11, pc[6]);
+    const float2 e0 = sub2(a10, a00), e1 = sub2(a11, a01);
+    const float2 b0 = fma2(fr[1], e0, a00), b1 = fma2(fr[1], e1, a01);
+    gz = sub2(b1, b0);
+    val = fma2(fr[2], gz, b0);
+    gy = lerp2(e0, e1, fr[2]);
+    gx = lerp2(lerp2(d00, d10, fr[1]), lerp2(d01, d11, fr[1]), fr[2]);
+}
+
+// The 8 corners of cell (cx, cy, cz) of the zero-bordered template (row pitch
+// MXP, MYP rows per plane, plane pitch SXYP).  Cells outside [-2, m] (padded
+// [0, m + 2]; CXM, CYM, CZM = m + 2) move to the far border, whose 8 corners
+// are zeros; so do the columns whose displacement is unusable (!ok).
+template <typename IMG>
+__device__ __forceinline__ void corners_padded(const IMG *T, int cx, int cy, int cz, bool ok, unsigned CXM, unsigned CYM,
+                                               unsigned CZM, int MXP, int MYP, size_t SXYP, float v[8])
+{
+    const unsigned ux = ok ? min((unsigned)cx, CXM) : CXM;
+    const unsigned uy = min((unsigned)cy, CYM), uz = min((unsigned)cz, CZM);
+    const IMG *p = T + ((size_t)(uy + (unsigned)MYP * uz) * MXP + ux);
+    v[0] = ldimg(p);
+    v[1] = ldimg(p + 1);
+    v[2] = ldimg(p + MXP);
+    v[3] = ldimg(p + MXP + 1);
+    v[4] = ldimg(p + SXYP);
+    v[5] = ldimg(p + SXYP + 1);
+    v[6] = ldimg(p + SXYP + MXP);
+    v[7] = ldimg(p + SXYP + MXP + 1);
+}
+
+// Phase B of a plane for a pair of columns from the ring of T~ planes (T0: the
+// pair's own entry of the plane, Tp and Tm of the planes above and below) and
+// R's normalized gradient field bn0, bn1 of the pair: (bx, bx'), (by, by') |
+// (bz, bz'), (rh, rh').  The x neighbours come from the threads beside it;
+// dyp, dym are the row steps (0 where the neighbour row is missing).
+__device__ __forceinline__ float2 ngf_pair_rn(const float *T0, const float *Tp, const float *Tm, int dyp, int dym,
+                                              const float4 &bn0, const float4 &bn1, float2 HX, float2 HY, float2 HZ,
+                                              float tau, float2 v[3])
+{
+    const float2 t0 = lds2(T0);
+    const float tl = __shfl_up_sync(0xffffffffu, t0.y, 1, BX);
+    const float tr = __shfl_down_sync(0xffffffffu, t0.x, 1, BX);
+    const float2 typ = lds2(T0 + dyp), tym = lds2(T0 - dym);
+    const float2 tzp = lds2(Tp), tzm = lds2(Tm);
+    const float2 av[3] = {mul2(make_float2(t0.y - tl, tr - t0.x), HX), mul2(sub2(typ, tym), HY),
+                          mul2(sub2(tzp, tzm), HZ)};
+    const float2 bh[3] = {make_float2(bn0.x, bn0.y), make_float2(bn0.z, bn0.w), make_float2(bn1.x, bn1.y)};
+    return ngf_residual_rn2(av, bh, make_float2(bn1.z, bn1.w), tau, v);
+}
+
+// Phase C: the adjoint of the central differences at a pair of columns from
+// the v rings (V0: the pair's v_x of the plane, v_y and v_z one and two PLANEs
+// on; Vzm, Vzp: v_z of the planes below and above), without the factor
+// hbar / 2.  vl, vr: v_x of the columns beside the pair.
+__device__ __forceinline__ float2 adjoint_pair(const float *V0, const float *Vzm, const float *Vzp, float2 vx, float vl,
+                                               float vr, float2 HX, float2 HY, float2 HZ)
+{
+    const float2 vyp = lds2(V0 + PLANE + CW), vym = lds2(V0 + PLANE - CW);
+    const float2 vzm = lds2(Vzm), vzp = lds2(Vzp);
+    return fma2(make_float2(vl - vx.y, vx.x - vr), HX, fma2(sub2(vym, vyp), HY, mul2(sub2(vzm, vzp), HZ)));
+}
+
 // Launch order of the tiles: the segment groups of the split by length,
 // longest first (so that the short tiles fill the SMs the long ones leave
 // free), then segment, then tile column.  Tile id -> (segment s in z order,
@@ -577,19 +648,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &a, int tile_id, floa
             const int cx = ix[k][0] + (k ? bx1 : bx0), cy = ix[k][1] + by, cz = ix[k][2] + bz;
             float v[8];
             if (PAD) {
-                // cells outside [-2, m] (padded [0, m + 2]) move to the far border, whose
-                // 8 corners are zeros; so do the columns whose displacement is unusable
-                const unsigned ux = okk ? min((unsigned)cx, CXM) : CXM;
-                const unsigned uy = min((unsigned)cy, CYM), uz = min((unsigned)cz, CZM);
-                const IMG *p = Tim + ((size_t)(uy + (unsigned)MYP * uz) * MXP + ux);
-                v[0] = ldimg(p);
-                v[1] = ldimg(p + 1);
-                v[2] = ldimg(p + MXP);
-                v[3] = ldimg(p + MXP + 1);
-                v[4] = ldimg(p + SXYP);
-                v[5] = ldimg(p + SXYP + 1);
-                v[6] = ldimg(p + SXYP + MXP);
-                v[7] = ldimg(p + SXYP + MXP + 1);
+                corners_padded(Tim, cx, cy, cz, okk, CXM, CYM, CZM, MXP, MYP, SXYP, v);
             } else {
 #pragma unroll
                 for (int j = 0; j < 8; j++)
@@ -633,17 +692,8 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &a, int tile_id, floa
         const int zA = z0 - 2 + s;
         // ---- A-finish: T~ and the interpolant differences on plane zA
         if (FULL || zA <= zend + 1) {
-            // corners: 0 = (0,0,0), 1 = (1,0,0), 2 = (0,1,0), 3 = (1,1,0), 4..7 the same at z + 1
-            const float2 d00 = sub2(pc[1], pc[0]), d10 = sub2(pc[3], pc[2]);
-            const float2 d01 = sub2(pc[5], pc[4]), d11 = sub2(pc[7], pc[6]);
-            const float2 a00 = fma2(fr[0], d00, pc[0]), a10 = fma2(fr[0], d10, pc[2]);
-            const float2 a01 = fma2(fr[0], d01, pc[4]), a11 = fma2(fr[0], d11, pc[6]);
-            const float2 e0 = sub2(a10, a00), e1 = sub2(a11, a01);
-            const float2 b0 = fma2(fr[1], e0, a00), b1 = fma2(fr[1], e1, a01);
-            const float2 gz = sub2(b1, b0);
-            const float2 val = fma2(fr[2], gz, b0);
-            const float2 gy = lerp2(e0, e1, fr[2]);
-            const float2 gx = lerp2(lerp2(d00, d10, fr[1]), lerp2(d01, d11, fr[1]), fr[2]);
+            float2 val, gx, gy, gz;
+            interp_pair(pc, fr, val, gx, gy, gz);
             const int slot = zA & 3;
             sts2(sm + SL::T + slot * PLANE + sp, val);
             if (!RN)
@@ -663,21 +713,10 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &a, int tile_id, floa
                 // R enters through its normalized gradient field, loaded a step ahead
                 // (zero off the interior and off the image): no interior tests, and
                 // rows 0 and BY - 1, whose v is never read, run the same code
-                const int o0 = (zB & 3) * PLANE + sp;
-                const float *T0 = sm + SL::T + o0;
-                const float2 t0 = lds2(T0);
-                const float tl = __shfl_up_sync(0xffffffffu, t0.y, 1, BX);
-                const float tr = __shfl_down_sync(0xffffffffu, t0.x, 1, BX);
-                const int op = ((zB + 1) & 3) * PLANE + sp, om = ((zB - 1) & 3) * PLANE + sp;
-                const float2 typ = lds2(T0 + dyp), tym = lds2(T0 - dym);
-                const float2 tzp = lds2(sm + SL::T + op), tzm = lds2(sm + SL::T + om);
-                const float2 av[3] = {mul2(make_float2(t0.y - tl, tr - t0.x), HX), mul2(sub2(typ, tym), HY),
-                                      mul2(sub2(tzp, tzm), HZ)};
-                // the field is stored by column pair: (bx, bx'), (by, by') | (bz, bz'), (rh, rh')
-                const float2 bh[3] = {make_float2(bn0.x, bn0.y), make_float2(bn0.z, bn0.w),
-                                      make_float2(bn1.x, bn1.y)};
+                const float *Tr = sm + SL::T + sp;
                 float2 v[3];
-                const float2 psi = ngf_residual_rn2(av, bh, make_float2(bn1.z, bn1.w), a.tau, v);
+                const float2 psi = ngf_pair_rn(Tr + (zB & 3) * PLANE, Tr + ((zB + 1) & 3) * PLANE,
+                                               Tr + ((zB - 1) & 3) * PLANE, dyp, dym, bn0, bn1, HX, HY, HZ, a.tau, v);
                 if (FULL || (zB >= z0 && zB < zend))
                     psi_sum.add(mul2(psi, MO));
                 float *vq = sm + SL::V + (zB & 3) * 3 * PLANE + sp;
@@ -741,11 +780,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &a, int tile_id, floa
             if (outxy && col_in && zC < mz) {
                 const float *Vzm = sm + SL::V + ((zC - 1) & 3) * 3 * PLANE + 2 * PLANE + sp;
                 const float *Vzp = sm + SL::V + ((zC + 1) & 3) * 3 * PLANE + 2 * PLANE + sp;
-                const float2 vyp = lds2(V0 + PLANE + CW), vym = lds2(V0 + PLANE - CW);
-                const float2 vzm = lds2(Vzm), vzp = lds2(Vzp);
-                // adjoint of the central differences (without the factor hbar / 2)
-                const float2 gj = fma2(make_float2(vl - vx.y, vx.x - vr), HX,
-                                       fma2(sub2(vym, vyp), HY, mul2(sub2(vzm, vzp), HZ)));
+                const float2 gj = adjoint_pair(V0, Vzm, Vzp, vx, vl, vr, HX, HY, HZ);
                 const float *gq = sm + SL::G + (gs == GSLOTS - 1 ? 0 : gs + 1) * 3 * PLANE + sp;
                 r[0] = mul2(gj, lds2(gq));
                 r[1] = mul2(gj, lds2(gq + PLANE));

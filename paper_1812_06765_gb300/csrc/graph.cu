@@ -206,6 +206,8 @@ int eval_kernel_count(const reg_ctx *c, int level)
         const Level &L = c->L[level];
         return (gather_blocks(L.n) < GATHER_SPLIT_BLOCKS ? 3 : 4) - (fused_curv_in_pass(c, level) ? 1 : 0);
     }
+    if (use_general(c, level))
+        return gather_blocks(c->L[level].n) < GATHER_SPLIT_BLOCKS ? 3 : 4;
     static const int ngf[3] = {4, 3, 10};   // multi-pass NGF kernels per P^T variant
     return ngf[mp_pt_variant(c, level)] + 3;   // + curvature, its gradient, final reduction
 }

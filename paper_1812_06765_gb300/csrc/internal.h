@@ -63,12 +63,13 @@ struct Level {
     double H[3];
     long long nv, nn;
     float *R = nullptr, *T = nullptr;        // device images
-    // read by the fused pass: T with a 2-voxel zero border on every side (dims m + 4), FP32
+    // read by the fused passes (general-ratio: FP32 always): T with a 2-voxel zero border on every side (dims m + 4), FP32
     // (image_dtype 0) or BF16 (Tb, image_dtype 1, beside the BF16 copy Rb of R)
     float *Tp = nullptr;
     __nv_bfloat16 *Rb = nullptr, *Tb = nullptr;
-    // read by the fused pass beside Tp: R's normalized gradient field (b / ||b||_rho,
-    // rho / ||b||_rho) per voxel, b the central-difference gradient; zero off the interior
+    // read by the fused passes beside Tp: R's normalized gradient field (b / ||b||_rho,
+    // rho / ||b||_rho) per voxel, b the central-difference gradient; zero off the interior;
+    // rows of an odd length carry one more column of zeros
     float4 *Rn = nullptr;
     int *pk0[3] = {nullptr, nullptr, nullptr};
     float *pw1[3] = {nullptr, nullptr, nullptr};
@@ -80,6 +81,7 @@ struct Level {
     int *qk0[3] = {nullptr, nullptr, nullptr};
     float *qw1[3] = {nullptr, nullptr, nullptr};
     FusedSplit split;   // z segments of the fused pass (not valid: not chosen yet)
+    FusedSplit gen_split;   // z segments of the general-ratio pass (any length)
     LevelGeom geom() const;
 };
 
@@ -227,6 +229,16 @@ cudaError_t launch_ngf_fused(reg_ctx *c, int level, const float *ub, const float
 cudaError_t launch_ngf_multipass(reg_ctx *c, int level, const float *ub, const float *dir, const double *t_dev,
                                  float *grad, double *partials, int *n_partials, cudaStream_t s);
 
+// the fused pass of grids of any ratio >= 2 voxels per node interval (k_ngf_general.cu)
+bool general_eligible(const Level &L);
+FusedSplit general_split(const int m[3], int num_sms);
+size_t general_part_floats(const Level &L);
+cudaError_t launch_ngf_general(reg_ctx *c, int level, const float *ub, const float *dir, const double *t_dev,
+                               int *n_partials, cudaStream_t s);
+// its node gather; fin: block 0 reduces J, D, S (and takes control phase >= 0) first
+cudaError_t launch_gather_general(reg_ctx *c, int level, const float *w, float alpha_hy, float *grad, bool fin, int nD,
+                                  const double *pS, int nS, double *scal, int phase, cudaStream_t s);
+
 cudaError_t launch_gather_grad(reg_ctx *c, int level, const float *w, float alpha_hy, float *grad, cudaStream_t s);
 // gather grids from this many blocks up run the final reduction beside the gather (side stream)
 constexpr long long GATHER_SPLIT_BLOCKS = 4096;
@@ -244,11 +256,19 @@ const void *curv_w_kernel();
 cudaError_t set_graph_kernel_priorities(cudaGraph_t g, const void *low_func);
 int eval_kernel_count(const reg_ctx *c, int level);
 
-// the fused pass serves levels whose grids have ratio exactly 2; others use the multi-pass kernels
+// the fused pass serves levels whose grids have ratio exactly 2, the general-ratio pass other
+// grids of ratio >= 2 (odd image sizes, quarter-resolution grids); denser node grids use the
+// multi-pass kernels
 inline bool use_fused(const reg_ctx *c, int level)
 {
     return c->cfg.eval_impl == 0 && fused_eligible(c->L[level]);
 }
+inline bool use_general(const reg_ctx *c, int level)
+{
+    return c->cfg.eval_impl == 0 && !fused_eligible(c->L[level]) && general_eligible(c->L[level]);
+}
+// voxels of R's normalized gradient field (rows of an even length)
+inline long long rn_voxels(const int m[3]) { return (long long)((m[0] + 1) & ~1) * m[1] * m[2]; }
 
 // Levels of at most WHOLE_LEVEL_MAX_NODES nodes are small: a level graph runs
 // them as one cooperative kernel (every iteration of the level, a grid barrier

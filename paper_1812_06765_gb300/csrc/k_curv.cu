@@ -127,7 +127,7 @@ cudaError_t launch_eval(reg_ctx *c, int level, const float *ub, const float *dir
     LevelGeom g = L.geom();
     int nD = 0;
     cudaError_t e;
-    const bool fused = use_fused(c, level);
+    const bool fused = use_fused(c, level), general = use_general(c, level);
     const bool curv_in_pass = fused && fused_curv_in_pass(c, level);
     // The curvature Laplacian (node pass, HBM-light) runs on the side stream
     // beside the NGF pass (issue-bound, one CTA per SM), in the tail of its last
@@ -144,6 +144,8 @@ cudaError_t launch_eval(reg_ctx *c, int level, const float *ub, const float *dir
     if (e == cudaSuccess) {
         if (fused)
             e = launch_ngf_fused(c, level, ub, dir, t_dev, grad, c->es.partials, &nD, s);
+        else if (general)
+            e = launch_ngf_general(c, level, ub, dir, t_dev, &nD, s);
         else
             e = launch_ngf_multipass(c, level, ub, dir, t_dev, grad, c->es.partials, &nD, s);
     }
@@ -173,10 +175,13 @@ cudaError_t launch_eval(reg_ctx *c, int level, const float *ub, const float *dir
     // gradient.  On small grids block 0 of the gather runs it first (one launch); on
     // large ones it is a one-block kernel on the side stream beside the gather, since
     // the control code in the gather would cost the large grid occupancy.
+    if (general && gather_blocks(L.n) < GATHER_SPLIT_BLOCKS)
+        return launch_gather_general(c, level, c->es.w, (float)(c->cfg.alpha * hy), grad, true, nD, pS, nS, scal_out,
+                                     ctl_phase, s);
     if (fused && gather_blocks(L.n) < GATHER_SPLIT_BLOCKS)
         return launch_gather_fin(c, level, c->es.w, (float)(c->cfg.alpha * hy), grad, nD, pS, nS, scal_out,
                                  ctl_phase, s);
-    if (fused) {
+    if (fused || general) {
         const double hbar = L.h[0] * L.h[1] * L.h[2];
         e = cudaEventRecord(c->ev_fork, s);
         if (e == cudaSuccess)
@@ -192,7 +197,10 @@ cudaError_t launch_eval(reg_ctx *c, int level, const float *ub, const float *dir
             }
             c->launches += 1;
         }
-        if (e == cudaSuccess)
+        if (e == cudaSuccess && general)
+            e = launch_gather_general(c, level, c->es.w, (float)(c->cfg.alpha * hy), grad, false, 0, nullptr, 0,
+                                      nullptr, -1, s);
+        else if (e == cudaSuccess)
             e = launch_gather_grad(c, level, c->es.w, (float)(c->cfg.alpha * hy), grad, s);
         if (e == cudaSuccess)
             e = cudaEventRecord(c->ev_join, c->side);

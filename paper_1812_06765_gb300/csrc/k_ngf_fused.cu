@@ -204,6 +204,29 @@ struct SplitModel {
             for (int tx = 0; tx < ntx; tx++)
                 colw.push_back(0.35 + 0.65 * frac(tx, OX, CW, m[0]) * frac(ty, OY, BY, m[1]));
     }
+    // the same with every column at weight 1, in pipeline steps: slots that fall free
+    // at the same time take tiles of the same length together
+    long long equal_columns(const FusedSplit &sp) const
+    {
+        int len[3] = {sp.l1, sp.l2, sp.lr}, cnt[3] = {sp.n1, sp.n2, sp.lr > 0 ? 1 : 0};
+        int ord[3] = {0, 1, 2};
+        std::stable_sort(ord, ord + 3, [&](int x, int y) { return len[x] > len[y]; });
+        std::map<long long, long long> free_at{{0, sms}};   // time -> slots
+        long long end = 0;
+        for (int k = 0; k < 3; k++)
+            for (long long tiles = (long long)cnt[ord[k]] * (long long)colw.size(); tiles > 0;) {
+                const auto it = free_at.begin();
+                const long long take = std::min(tiles, it->second), t = it->first + len[ord[k]] + FUSED_FILL;
+                if (it->second == take)
+                    free_at.erase(it);
+                else
+                    it->second -= take;
+                free_at[t] += take;
+                tiles -= take;
+                end = std::max(end, t);
+            }
+        return end;
+    }
     double makespan(const FusedSplit &sp) const
     {
         // segment groups by length, longest first (stable), as tile_seg_col
@@ -269,6 +292,47 @@ static std::vector<FusedSplit> splits_ranked(const int m[3], int num_sms)
     for (auto &e : r)
         v.push_back(e.second);
     return v;
+}
+
+// Split of the general-ratio pass (k_ngf_general.cu): the load model's choice
+// without a timing run or a replay of every candidate (tens of milliseconds,
+// which a geometry used once would pay).  All candidates are ranked with equal
+// tile columns, whose replay moves groups of slots that fall free together;
+// the best few are then replayed tile by tile.  Cached per dims.
+FusedSplit general_split(const int m[3], int num_sms)
+{
+    constexpr int REPLAYED = 8;
+    static std::mutex mu;
+    static std::map<std::array<int, 4>, FusedSplit> cache;
+    const std::array<int, 4> key{m[0], m[1], m[2], num_sms};
+    {
+        std::lock_guard<std::mutex> lk(mu);
+        auto it = cache.find(key);
+        if (it != cache.end())
+            return it->second;
+    }
+    const SplitModel model(m, num_sms);
+    std::vector<std::pair<long long, FusedSplit>> r;
+    for (const FusedSplit &sp : split_candidates(m[2]))
+        r.push_back({model.equal_columns(sp), sp});
+    std::stable_sort(r.begin(), r.end(),
+                     [](const std::pair<long long, FusedSplit> &x, const std::pair<long long, FusedSplit> &y) {
+                         return x.first != y.first ? x.first < y.first : x.second.count() < y.second.count();
+                     });
+    FusedSplit best;
+    double best_t = 0.0;
+    for (size_t i = 0; i < r.size() && i < REPLAYED; i++) {
+        const double t = model.makespan(r[i].second);
+        if (!best.valid() || t < best_t) {
+            best = r[i].second;
+            best_t = t;
+        }
+    }
+    std::lock_guard<std::mutex> lk(mu);
+    if (cache.size() >= 4096)   // a long-lived process with ever new geometries
+        cache.clear();
+    cache[key] = best;
+    return best;
 }
 
 FusedSplit fused_split(const Level &L, int num_sms) { return L.split.valid() ? L.split : splits_ranked(L.m, num_sms)[0]; }

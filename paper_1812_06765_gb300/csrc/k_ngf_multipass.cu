@@ -1,7 +1,8 @@
 // Multi-pass objective evaluation: one kernel per step of Sec. 2.2
-// "Evaluating the objective function", intermediates in HBM.  It is the
-// plain-structured variant kept beside the fused pass (reg_config.eval_impl =
-// 1), used to cross-check it and as the A/B baseline for its traffic.
+// "Evaluating the objective function", intermediates in HBM.  It serves grids
+// of less than 2 voxels per node interval, and is the plain-structured variant
+// kept beside the fused passes (reg_config.eval_impl = 1), used to cross-check
+// them and as the A/B baseline for their traffic.
 //
 //   k_mp_warp   : y-hat = P u (Eq. 1), T(x + y-hat) and the interpolant gradient
 //   k_mp_resid  : NGF residual on interior voxels (Eq. 2), v = d psi / d grad T

@@ -104,15 +104,17 @@ __global__ void __launch_bounds__(256) k_pad_template(const float *__restrict__ 
 // Stored by pairs of columns (x even, x + 1: the two columns a thread of the
 // pass holds), 8 floats per pair: bx, bx', by, by' | bz, bz', rho', rho'',
 // so that every pair of lanes of the pass's packed arithmetic is one 8-byte
-// half of a 16-byte load.  The row length is even, so pair p of a row starts
-// at float 8 p and the array has 4 floats per voxel, as a float4 per voxel.
+// half of a 16-byte load.  The row length is rounded up to even, so pair p of
+// a row starts at float 8 p and the array has 4 floats per voxel of such rows,
+// as a float4 per voxel.
 __global__ void k_ref_normal_field(const float *__restrict__ R, int mx, int my, int mz, float hx, float hy, float hz,
                                    float rho, float4 *__restrict__ out)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
     const int y = blockIdx.y * blockDim.y + threadIdx.y;
     const int z = blockIdx.z;
-    if (x >= mx || y >= my)
+    const int mxe = (mx + 1) & ~1;   // rows of an odd length carry one more column of zeros
+    if (x >= mxe || y >= my)
         return;
     const size_t sy = (size_t)mx, sz = (size_t)mx * my;
     const size_t i = x + sy * y + sz * z;
@@ -127,7 +129,8 @@ __global__ void k_ref_normal_field(const float *__restrict__ R, int mx, int my, 
         o[2] = bz / nb;
         o[3] = rho / nb;
     }
-    float *pair = reinterpret_cast<float *>(out) + 4 * (i - (x & 1));   // 8 floats of the column pair
+    // 8 floats of the column pair
+    float *pair = reinterpret_cast<float *>(out) + 4 * ((x & ~1) + (size_t)mxe * (y + (size_t)my * z));
 #pragma unroll
     for (int c = 0; c < 4; c++)
         pair[2 * c + (x & 1)] = o[c];
@@ -161,7 +164,7 @@ cudaError_t launch_ref_normal_field(const Level &L, double rho, cudaStream_t s)
     // the pass's difference factors: 0.5 * (float)(1 / h), as in grad T~
     const LevelGeom g = L.geom();
     dim3 blk(32, 8, 1);
-    dim3 grd((L.m[0] + 31) / 32, (L.m[1] + 7) / 8, L.m[2]);
+    dim3 grd((L.m[0] + 32) / 32, (L.m[1] + 7) / 8, L.m[2]);   // an odd row's extra column included
     k_ref_normal_field<<<grd, blk, 0, s>>>(L.R, L.m[0], L.m[1], L.m[2], 0.5f * g.ih[0], 0.5f * g.ih[1],
                                            0.5f * g.ih[2], (float)rho, L.Rn);
     return cudaGetLastError();

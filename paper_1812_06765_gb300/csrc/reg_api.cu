@@ -279,6 +279,10 @@ int allocate_buffers(reg_ctx *c)
         if (use_fused(c, l)) {
             size_t p = fused_part_floats(c->L[l], c->num_sms);
             if (p > part) part = p;
+        } else if (use_general(c, l)) {
+            c->L[l].gen_split = general_split(c->L[l].m, c->num_sms);
+            size_t p = general_part_floats(c->L[l]);
+            if (p > part) part = p;
         } else if (c->L[l].nv > mp_vox) {
             mp_vox = c->L[l].nv;
         }
@@ -293,16 +297,16 @@ int allocate_buffers(reg_ctx *c)
         CK(cudaMalloc(&es.part, sizeof(float) * part));
         es.part_floats = part;
     }
-    // the fused pass reads T through a zero-bordered copy (FP32, or BF16 beside a BF16 R)
+    // the fused passes read T through a zero-bordered copy (FP32, or BF16 beside a BF16 R)
     for (int l = 0; l < c->levels; l++)
-        if (use_fused(c, l)) {
+        if (use_fused(c, l) || use_general(c, l)) {
             const long long np = padded_voxels(c->L[l].m);
-            if (cfg.image_dtype == 1) {
+            if (cfg.image_dtype == 1 && use_fused(c, l)) {
                 CK(cudaMalloc(&c->L[l].Rb, sizeof(__nv_bfloat16) * c->L[l].nv));
                 CK(cudaMalloc(&c->L[l].Tb, sizeof(__nv_bfloat16) * np));
             } else {
                 CK(cudaMalloc(&c->L[l].Tp, sizeof(float) * np));
-                CK(cudaMalloc(&c->L[l].Rn, sizeof(float4) * c->L[l].nv));
+                CK(cudaMalloc(&c->L[l].Rn, sizeof(float4) * rn_voxels(c->L[l].m)));
             }
         }
     CK(cudaMalloc(&es.w, sizeof(float) * nmax));
