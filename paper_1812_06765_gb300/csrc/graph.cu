@@ -69,13 +69,12 @@ cudaError_t add_while(cudaGraph_t g, const std::vector<cudaGraphNode_t> &deps, c
 }  // namespace
 
 // Kernel node priorities of one graph (not its conditional bodies): the
-// kernel low_func (the curvature Laplacian, which runs beside the NGF pass) at
-// the device's lowest stream priority and every other kernel at the highest,
+// curvature Laplacian, which runs beside the NGF pass, at the device's lowest stream priority and every other kernel at the highest,
 // so that the block scheduler hands out the NGF pass's CTAs (one per SM) first
 // and the curvature blocks take the SMs that the NGF pass's last, shorter tiles
 // leave idle.  The graph must be instantiated with
 // cudaGraphInstantiateFlagUseNodePriority for the priorities to apply.
-cudaError_t set_graph_kernel_priorities(cudaGraph_t g, const void *low_func)
+cudaError_t set_graph_kernel_priorities(cudaGraph_t g)
 {
     int lowest = 0, highest = 0;
     cudaError_t e = cudaDeviceGetStreamPriorityRange(&lowest, &highest);
@@ -96,7 +95,7 @@ cudaError_t set_graph_kernel_priorities(cudaGraph_t g, const void *low_func)
         if (e != cudaSuccess)
             break;
         cudaLaunchAttributeValue v = {};
-        v.priority = kp.func == low_func ? lowest : highest;
+        v.priority = is_curv_w_kernel(kp.func) ? lowest : highest;
         e = cudaGraphKernelNodeSetAttribute(nodes[i], cudaLaunchAttributePriority, &v);
     }
     return e;
@@ -192,7 +191,7 @@ cudaError_t build_level_graph(reg_ctx *c, int level, cudaGraphExec_t *out)
     }
     lbfgs_set_graph_handles(0, 0, 0);
     for (cudaGraph_t g : {G, body, redo_body, ls_body})
-        GK(set_graph_kernel_priorities(g, curv_w_kernel()));
+        GK(set_graph_kernel_priorities(g));
     GK(cudaGraphInstantiate(out, G, cudaGraphInstantiateFlagUseNodePriority));
     cudaGraphDestroy(G);
     c->launches = launches0;

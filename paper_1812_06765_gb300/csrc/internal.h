@@ -153,10 +153,15 @@ int cuda_err(reg_ctx *c, cudaError_t e, const char *what);
         if (_e != cudaSuccess) return cuda_err(c, _e, #call);             \
     } while (0)
 
-// The curvature Laplacian pass: blocks of 32 x 8 nodes over CURV_ZB node
-// planes, one FP64 partial of S per block.
-#define CURV_ZB 1
-inline int curv_zchunks(int nz) { return (nz + CURV_ZB - 1) / CURV_ZB; }
+// The curvature Laplacian pass: blocks of CURV_NODES consecutive nodes of a node
+// plane on curv_planes() node planes, one FP64 partial of S per block.  A thread
+// marches through as many planes (up to 4) as leave 2048 blocks, a few resident waves.
+constexpr int CURV_NODES = 256;
+inline int curv_planes(const int n[3])
+{
+    const long long p = (long long)n[0] * n[1] * n[2] / (CURV_NODES * 2048LL);
+    return p < 1 ? 1 : p > 4 ? 4 : (int)p;
+}
 
 // launchers (return cudaError_t of the launch)
 cudaError_t launch_restrict(const float *src, const int m[3], float *dst, cudaStream_t s);
@@ -250,10 +255,10 @@ inline dim3 gather_grid(const int n[3]) { return dim3(gather_runs_per_plane(n), 
 inline long long gather_blocks(const int n[3]) { return (long long)gather_runs_per_plane(n) * n[2]; }
 
 cudaError_t build_level_graph(reg_ctx *c, int level, cudaGraphExec_t *out);
-// the curvature Laplacian kernels that run beside the NGF pass (to tell their graph nodes apart)
-const void *curv_w_kernel();
-// kernel nodes of g: low_func at the lowest priority, the others at the highest
-cudaError_t set_graph_kernel_priorities(cudaGraph_t g, const void *low_func);
+// whether f is a curvature Laplacian kernel, which runs beside the NGF pass (to tell their graph nodes apart)
+bool is_curv_w_kernel(const void *f);
+// kernel nodes of g: the curvature Laplacian at the lowest priority, the others at the highest
+cudaError_t set_graph_kernel_priorities(cudaGraph_t g);
 int eval_kernel_count(const reg_ctx *c, int level);
 
 // the fused pass serves levels whose grids have ratio exactly 2, the general-ratio pass other

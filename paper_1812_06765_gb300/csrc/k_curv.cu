@@ -12,52 +12,80 @@
 
 namespace {
 
-// block (bx, by, bzc) of 32 x 8 nodes over the CURV_ZB node planes from
-// bzc * CURV_ZB; its S partial goes to partials[lin]
-__device__ __forceinline__ void curv_w_body(const LevelGeom &g, const float *__restrict__ ub,
-                                            const float *__restrict__ dir, const double *__restrict__ t_dev,
-                                            float *__restrict__ w, double *__restrict__ partials, int bx, int by,
-                                            int bzc, int lin)
+// element at a 32-bit byte offset from a base that is the same for the whole
+// grid: one address register instead of 64-bit arithmetic per load (a plane
+// array of one component holds less than 2^32 bytes, as 3 hold < 2^31 elements)
+__device__ __forceinline__ float ld_at(const float *base, unsigned byte)
 {
-    __shared__ double sm[8];
-    const int x = bx * blockDim.x + threadIdx.x;
-    const int y = by * blockDim.y + threadIdx.y;
-    const bool in = x < g.n[0] && y < g.n[1];
-    const float t = dir ? (float)__ldg(t_dev) : 0.f;
-    const size_t st[3] = {1, (size_t)g.n[0], (size_t)g.n[0] * g.n[1]};
-    const bool inxy = x >= 1 && y >= 1 && x <= g.n[0] - 2 && y <= g.n[1] - 2;
-    const int z1 = min(g.n[2], (bzc + 1) * CURV_ZB);
-    float acc = 0.f;
-    if (in)
-        for (int z = bzc * CURV_ZB; z < z1; z++) {
-            const size_t k = x + (size_t)g.n[0] * (y + (size_t)g.n[1] * z);
-            const bool interior = inxy && z >= 1 && z <= g.n[2] - 2;
-#pragma unroll
-            for (int c = 0; c < 3; c++) {
-                float lap = 0.f;
-                if (interior) {
-                    const float *u = ub + c * g.nn;
-                    const float *d = dir ? dir + c * g.nn : nullptr;
-                    float u0 = node_value(u, d, t, k);
-#pragma unroll
-                    for (int e = 0; e < 3; e++)
-                        lap = fmaf(node_value(u, d, t, k + st[e]) - 2.f * u0 + node_value(u, d, t, k - st[e]),
-                                   g.iH2[e], lap);
-                }
-                w[c * g.nn + k] = lap;
-                acc = fmaf(lap, lap, acc);
-            }
-        }
-    double s = block_sum_to_f64(acc, sm);
-    if (linear_tid() == 0)
-        partials[lin] = s;
+    return __ldg(reinterpret_cast<const float *>(reinterpret_cast<const char *>(base) + byte));
 }
 
-__global__ void __launch_bounds__(256) k_curv_w(LevelGeom g, const float *__restrict__ ub,
-                                                const float *__restrict__ dir, const double *__restrict__ t_dev,
-                                                float *__restrict__ w, double *__restrict__ partials)
+// A block takes CURV_NODES consecutive nodes of a plane (no lane idles at the
+// end of a row) on curv_planes() node planes.  The z neighbours move up through
+// registers, the x and y ones come from L1 at 32-bit offsets (a border node's
+// missing neighbour reads the node itself; its w is masked).  HAS_DIR: at
+// u + t dir.  The NGF pass's CTAs hold the whole register file, so this kernel
+// runs before them or in their tail, and its time counts: 129^3 nodes 28 ->
+// 19.5 us, 371 -> 154 instructions a node (one plane of 32 x 8 nodes a block,
+// 64-bit addresses).  Past 4 planes a thread the gain is gone: fewer blocks
+// than a wave or two.
+template <bool HAS_DIR>
+__global__ void __launch_bounds__(CURV_NODES) k_curv_w(LevelGeom g, const float *__restrict__ ub,
+                                                         const float *__restrict__ dir,
+                                                         const double *__restrict__ t_dev, float *__restrict__ w,
+                                                         double *__restrict__ partials, int planes)
 {
-    curv_w_body(g, ub, dir, t_dev, w, partials, blockIdx.x, blockIdx.y, blockIdx.z, linear_bid());
+    __shared__ double sm[8];
+    const int n0 = g.n[0];
+    const int i = blockIdx.x * CURV_NODES + threadIdx.x;
+    const int z0 = blockIdx.y * planes, z1 = min(g.n[2], z0 + planes);
+    const float t = HAS_DIR ? (float)__ldg(t_dev) : 0.f;
+    KahanF acc;
+    if (i < n0 * g.n[1]) {
+        const int y = i / n0, x = i - y * n0;
+        const bool inxy = x >= 1 && y >= 1 && x <= n0 - 2 && y <= g.n[1] - 2;
+        const unsigned plane = 4u * n0 * g.n[1];
+        unsigned o = 4u * i + plane * z0;
+        unsigned xm = inxy ? o - 4u : o, xp = inxy ? o + 4u : o;
+        unsigned ym = inxy ? o - 4u * n0 : o, yp = inxy ? o + 4u * n0 : o;
+        // the trial value, as the accepted update forms it
+        auto node = [&](int d, unsigned b) {
+            const float v = ld_at(ub + d * g.nn, b);
+            return HAS_DIR ? fmaf(t, ld_at(dir + d * g.nn, b), v) : v;
+        };
+        float m[3], c[3];
+#pragma unroll
+        for (int d = 0; d < 3; d++) {
+            m[d] = node(d, z0 > 0 ? o - plane : o);
+            c[d] = node(d, o);
+        }
+        for (int z = z0; z < z1; z++) {
+            const bool top = z == g.n[2] - 1, in = inxy && z >= 1 && !top;
+            const unsigned up = top ? o : o + plane;
+            float sq = 0.f;
+#pragma unroll
+            for (int d = 0; d < 3; d++) {
+                const float p = node(d, up);
+                float lap = fmaf(node(d, xp) - 2.f * c[d] + node(d, xm), g.iH2[0], 0.f);
+                lap = fmaf(node(d, yp) - 2.f * c[d] + node(d, ym), g.iH2[1], lap);
+                lap = fmaf(p - 2.f * c[d] + m[d], g.iH2[2], lap);
+                lap = in ? lap : 0.f;
+                *reinterpret_cast<float *>(reinterpret_cast<char *>(w + d * g.nn) + o) = lap;
+                sq = fmaf(lap, lap, sq);
+                m[d] = c[d];
+                c[d] = p;
+            }
+            acc.add(sq);
+            o += plane;
+            xm += plane;
+            xp += plane;
+            ym += plane;
+            yp += plane;
+        }
+    }
+    const double s = block_sum_to_f64(acc.s, sm);
+    if (linear_tid() == 0)
+        partials[linear_bid()] = s;
 }
 
 __global__ void __launch_bounds__(256) k_curv_grad(LevelGeom g, const float *__restrict__ w, float alpha_hy,
@@ -111,7 +139,10 @@ __global__ void __launch_bounds__(512) k_finalize_batch(const PairLevel *__restr
 
 }  // namespace
 
-const void *curv_w_kernel() { return reinterpret_cast<const void *>(k_curv_w); }
+bool is_curv_w_kernel(const void *f)
+{
+    return f == reinterpret_cast<const void *>(k_curv_w<true>) || f == reinterpret_cast<const void *>(k_curv_w<false>);
+}
 
 
 cudaError_t launch_finalize_batch(const PairLevel *pl, int npairs, int mode, cudaStream_t s)
@@ -155,10 +186,12 @@ cudaError_t launch_eval(reg_ctx *c, int level, const float *ub, const float *dir
         return e;
     dim3 blk(32, 8, 1);
     dim3 gn((L.n[0] + 31) / 32, (L.n[1] + 7) / 8, L.n[2]);
-    dim3 gw(gn.x, gn.y, curv_zchunks(L.n[2]));
+    const int planes = curv_planes(L.n);
+    const dim3 gw((L.n[0] * L.n[1] + CURV_NODES - 1) / CURV_NODES, (L.n[2] + planes - 1) / planes, 1);
     double *pS = c->es.partials + nD;
     if (!curv_in_pass) {
-        k_curv_w<<<gw, blk, 0, c->side>>>(g, ub, dir, t_dev, c->es.w, pS);
+        dir ? k_curv_w<true><<<gw, CURV_NODES, 0, c->side>>>(g, ub, dir, t_dev, c->es.w, pS, planes)
+            : k_curv_w<false><<<gw, CURV_NODES, 0, c->side>>>(g, ub, dir, t_dev, c->es.w, pS, planes);
         c->launches += 1;
         e = cudaGetLastError();
     }
