@@ -34,7 +34,7 @@ void fill_pair_level(reg_ctx *c, int level, PairLevel &P)
     a.g = P.geom;
     a.T = bf16 ? static_cast<const void *>(L.Tb) : static_cast<const void *>(L.Tp);   // zero-bordered copies
     a.R = bf16 ? static_cast<const void *>(L.Rb) : static_cast<const void *>(L.R);
-    a.Rn = bf16 ? nullptr : L.Rn;   // R's normalized gradient field (FP32 images)
+    a.Rn = L.Rn;
     a.ub = c->lb.u;
     a.dir = nullptr;
     a.t_dev = nullptr;

@@ -64,9 +64,10 @@ struct Level {
     long long nv, nn;
     float *R = nullptr, *T = nullptr;        // device images
     // read by the fused passes (general-ratio: FP32 always): T with a 2-voxel zero border on every side (dims m + 4), FP32
-    // (image_dtype 0) or BF16 (Tb, image_dtype 1, beside the BF16 copy Rb of R)
+    // (image_dtype 0) or BF16 x pairs (Tb, image_dtype 1, beside the BF16 copy Rb of R)
     float *Tp = nullptr;
-    __nv_bfloat16 *Rb = nullptr, *Tb = nullptr;
+    __nv_bfloat16 *Rb = nullptr;
+    __nv_bfloat162 *Tb = nullptr;
     // read by the fused passes beside Tp: R's normalized gradient field (b / ||b||_rho,
     // rho / ||b||_rho) per voxel, b the central-difference gradient; zero off the interior;
     // rows of an odd length carry one more column of zeros
@@ -169,7 +170,9 @@ cudaError_t launch_to_bf16(const float *src, __nv_bfloat16 *dst, long long n, cu
 // the zero-bordered copy of a volume of dims m read by the fused pass (dims m + 4)
 long long padded_voxels(const int m[3]);
 cudaError_t launch_pad_template(const float *src, const int m[3], float *dst, cudaStream_t s);
-cudaError_t launch_pad_template(const float *src, const int m[3], __nv_bfloat16 *dst, cudaStream_t s);
+// BF16: element x holds (T[x], T[x + 1])
+cudaError_t launch_pad_template(const float *src, const int m[3], __nv_bfloat162 *dst, cudaStream_t s);
+// of R, or of R rounded to BF16 (its copy L.Rb)
 cudaError_t launch_ref_normal_field(const Level &L, double rho, cudaStream_t s);
 cudaError_t launch_prolong(const Level &coarse, const Level &fine, const float *uc, float *uf, cudaStream_t s);
 

@@ -391,7 +391,7 @@ FusedArgs fused_args(const reg_ctx *c, int level, const float *ub, const float *
     const bool bf16 = c->cfg.image_dtype == 1 && L.Tb && L.Rb;
     a.T = bf16 ? static_cast<const void *>(L.Tb) : static_cast<const void *>(L.Tp);   // zero-bordered copies
     a.R = bf16 ? L.Rb : static_cast<const void *>(L.R);
-    a.Rn = bf16 ? nullptr : L.Rn;
+    a.Rn = L.Rn;
     a.ub = ub;
     a.dir = dir;
     a.t_dev = t_dev;
@@ -414,8 +414,8 @@ cudaError_t launch_ngf_fused(reg_ctx *c, int level, const float *ub, const float
     (void)grad;
     const Level &L = c->L[level];
     const bool bf16 = c->cfg.image_dtype == 1 && L.Tb && L.Rb;
-    if (!bf16 && !L.Rn)
-        return cudaErrorInvalidValue;   // FP32 handles keep R's normalized field beside the padded T
+    if (!L.Rn)
+        return cudaErrorInvalidValue;   // handles keep R's normalized field beside the padded T
     int ntiles = 0;
     const FusedArgs a = fused_args(c, level, ub, dir, t_dev, partials, &ntiles);
     dim3 blk(BX, BY, 1), grd(ntiles, 1, 1);

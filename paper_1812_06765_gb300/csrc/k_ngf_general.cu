@@ -74,7 +74,7 @@ struct GSmem {
 
 struct GenArgs {
     LevelGeom g;
-    const float *T;         // zero-bordered template
+    const void *T;          // zero-bordered template
     const float4 *Rn;       // R's normalized gradient field (row length rounded up to even)
     const float *ub, *dir;
     const double *t_dev;
@@ -296,7 +296,7 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
 #pragma unroll
         for (int k = 0; k < 2; k++) {
             float v[8];
-            corners_padded(a.T, ix[k][0] + (k ? bx1 : bx0), ix[k][1] + by, ix[k][2] + bz + z1, k ? ok1 : ok0, CXM, CYM,
+            corners_padded(static_cast<const TemplateElem<float>::type *>(a.T), ix[k][0] + (k ? bx1 : bx0), ix[k][1] + by, ix[k][2] + bz + z1, k ? ok1 : ok0, CXM, CYM,
                            CZM, MXP, MYP, SXYP, v);
 #pragma unroll
             for (int j = 0; j < 8; j++) {

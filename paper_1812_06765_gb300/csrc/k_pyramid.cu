@@ -6,6 +6,8 @@
 // streams.  Prolongation (Sec. 2.1, coarse-to-fine): nodal trilinear
 // interpolation of the coarse displacement onto the finer nodes, with
 // per-dimension (first node, weight) tables.
+#include <type_traits>
+
 #include "internal.h"
 
 namespace {
@@ -74,8 +76,9 @@ __global__ void __launch_bounds__(256) k_to_bf16(const float *__restrict__ src, 
         dst[4 * n4 + threadIdx.x] = __float2bfloat16_rn(src[4 * n4 + threadIdx.x]);
 }
 
-__device__ __forceinline__ void pad_store(float *p, float v) { *p = v; }
-__device__ __forceinline__ void pad_store(__nv_bfloat16 *p, float v) { *p = __float2bfloat16_rn(v); }
+// element x of the padded array from the image's values at x and x + 1
+__device__ __forceinline__ void pad_store(float *p, float v, float) { *p = v; }
+__device__ __forceinline__ void pad_store(__nv_bfloat162 *p, float v, float vn) { *p = __floats2bfloat162_rn(v, vn); }
 
 // Zero-bordered copy of a volume (dims m) into an array of dims m + 4 with the
 // volume at offset 2 in every dimension: one thread per element of the
@@ -90,10 +93,16 @@ __global__ void __launch_bounds__(256) k_pad_template(const float *__restrict__ 
     if (x >= px || y >= py)
         return;
     const int sx = x - 2, sy = y - 2, sz = z - 2;
-    const bool in = (unsigned)sx < (unsigned)mx && (unsigned)sy < (unsigned)my && (unsigned)sz < (unsigned)mz;
-    const float v = in ? __ldg(src + ((size_t)sz * my + sy) * mx + sx) : 0.f;
-    pad_store(dst + ((size_t)z * py + y) * px + x, v);
+    const bool in = (unsigned)sy < (unsigned)my && (unsigned)sz < (unsigned)mz;
+    const float *row = src + ((size_t)sz * my + sy) * mx;
+    const float v = in && (unsigned)sx < (unsigned)mx ? __ldg(row + sx) : 0.f;
+    const bool pairs = !std::is_same<TOUT, float>::value;
+    const float vn = pairs && in && (unsigned)(sx + 1) < (unsigned)mx ? __ldg(row + sx + 1) : 0.f;
+    pad_store(dst + ((size_t)z * py + y) * px + x, v, vn);
 }
+
+__device__ __forceinline__ float ld_img(const float *p) { return __ldg(p); }
+__device__ __forceinline__ float ld_img(const __nv_bfloat16 *p) { return __bfloat162float(__ldg(p)); }
 
 // R's normalized gradient field for the fused pass (Eq. 2): R is fixed for the
 // whole registration, so its part of every NGF term is formed once per level.
@@ -107,7 +116,8 @@ __global__ void __launch_bounds__(256) k_pad_template(const float *__restrict__ 
 // half of a 16-byte load.  The row length is rounded up to even, so pair p of
 // a row starts at float 8 p and the array has 4 floats per voxel of such rows,
 // as a float4 per voxel.
-__global__ void k_ref_normal_field(const float *__restrict__ R, int mx, int my, int mz, float hx, float hy, float hz,
+template <typename TIN>
+__global__ void k_ref_normal_field(const TIN *__restrict__ R, int mx, int my, int mz, float hx, float hy, float hz,
                                    float rho, float4 *__restrict__ out)
 {
     const int x = blockIdx.x * blockDim.x + threadIdx.x;
@@ -120,9 +130,9 @@ __global__ void k_ref_normal_field(const float *__restrict__ R, int mx, int my, 
     const size_t i = x + sy * y + sz * z;
     float o[4] = {0.f, 0.f, 0.f, 0.f};
     if (x >= 1 && x <= mx - 2 && y >= 1 && y <= my - 2 && z >= 1 && z <= mz - 2) {
-        const float bx = (__ldg(R + i + 1) - __ldg(R + i - 1)) * hx;
-        const float by = (__ldg(R + i + sy) - __ldg(R + i - sy)) * hy;
-        const float bz = (__ldg(R + i + sz) - __ldg(R + i - sz)) * hz;
+        const float bx = (ld_img(R + i + 1) - ld_img(R + i - 1)) * hx;
+        const float by = (ld_img(R + i + sy) - ld_img(R + i - sy)) * hy;
+        const float bz = (ld_img(R + i + sz) - ld_img(R + i - sz)) * hz;
         const float nb = sqrtf(fmaf(bz, bz, fmaf(by, by, bx * bx)) + rho * rho);
         o[0] = bx / nb;
         o[1] = by / nb;
@@ -154,7 +164,7 @@ cudaError_t launch_pad_template(const float *src, const int m[3], float *dst, cu
     return launch_pad(src, m, dst, s);
 }
 
-cudaError_t launch_pad_template(const float *src, const int m[3], __nv_bfloat16 *dst, cudaStream_t s)
+cudaError_t launch_pad_template(const float *src, const int m[3], __nv_bfloat162 *dst, cudaStream_t s)
 {
     return launch_pad(src, m, dst, s);
 }
@@ -165,8 +175,11 @@ cudaError_t launch_ref_normal_field(const Level &L, double rho, cudaStream_t s)
     const LevelGeom g = L.geom();
     dim3 blk(32, 8, 1);
     dim3 grd((L.m[0] + 32) / 32, (L.m[1] + 7) / 8, L.m[2]);   // an odd row's extra column included
-    k_ref_normal_field<<<grd, blk, 0, s>>>(L.R, L.m[0], L.m[1], L.m[2], 0.5f * g.ih[0], 0.5f * g.ih[1],
-                                           0.5f * g.ih[2], (float)rho, L.Rn);
+    const float hx = 0.5f * g.ih[0], hy = 0.5f * g.ih[1], hz = 0.5f * g.ih[2];
+    if (L.Rb)
+        k_ref_normal_field<<<grd, blk, 0, s>>>(L.Rb, L.m[0], L.m[1], L.m[2], hx, hy, hz, (float)rho, L.Rn);
+    else
+        k_ref_normal_field<<<grd, blk, 0, s>>>(L.R, L.m[0], L.m[1], L.m[2], hx, hy, hz, (float)rho, L.Rn);
     return cudaGetLastError();
 }
 

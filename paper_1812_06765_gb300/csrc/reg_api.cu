@@ -303,11 +303,11 @@ int allocate_buffers(reg_ctx *c)
             const long long np = padded_voxels(c->L[l].m);
             if (cfg.image_dtype == 1 && use_fused(c, l)) {
                 CK(cudaMalloc(&c->L[l].Rb, sizeof(__nv_bfloat16) * c->L[l].nv));
-                CK(cudaMalloc(&c->L[l].Tb, sizeof(__nv_bfloat16) * np));
+                CK(cudaMalloc(&c->L[l].Tb, sizeof(__nv_bfloat162) * np));
             } else {
                 CK(cudaMalloc(&c->L[l].Tp, sizeof(float) * np));
-                CK(cudaMalloc(&c->L[l].Rn, sizeof(float4) * rn_voxels(c->L[l].m)));
             }
+            CK(cudaMalloc(&c->L[l].Rn, sizeof(float4) * rn_voxels(c->L[l].m)));
         }
     CK(cudaMalloc(&es.w, sizeof(float) * nmax));
     CK(cudaMalloc(&es.partials, sizeof(double) * maxpart));
@@ -501,8 +501,11 @@ int reg_set_images(reg_handle c, const float *R, const float *T, const int dims[
         }
         if (c->L[l].Tp) {
             CK(launch_pad_template(c->L[l].T, c->L[l].m, c->L[l].Tp, c->stream));
+            c->launches += 1;
+        }
+        if (c->L[l].Rn) {
             CK(launch_ref_normal_field(c->L[l], cfg.rho, c->stream));
-            c->launches += 2;
+            c->launches += 1;
         }
     }
     // tiling of the fused pass per level: forced, autotuned (at u = 0, with the
