@@ -9,7 +9,7 @@
 // gradient field.  What differs:
 //   P      the weights of a column and the nodes it lies between come from the
 //          tables; the pair's columns lie in the same node interval or in
-//          adjacent ones, so one 3 x 2 block of nodes serves both.  A plane
+//          adjacent ones, so one 3 x 2 x 2 block of nodes serves both.  A plane
 //          takes its weight from the table along z, and the block's node
 //          planes advance when the plane's interval does (at most every other
 //          plane at 2 voxels per interval).
@@ -155,14 +155,9 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
     }
     // the pair's node intervals: the second column lies in the first's or the next one
     const int lkx = kxs[2 * tx] - kx0, lky = kys[ty] - ky0;
-    float2 C1, C2, WYv;
-    {
-        const float wa = sm[SL::WX + 2 * tx], wb = sm[SL::WX + 2 * tx + 1];
-        const bool next = kxs[2 * tx + 1] != kxs[2 * tx];
-        C1 = make_float2(wa, next ? 1.f : wb);
-        C2 = make_float2(0.f, next ? wb : 0.f);
-        WYv = bc2(sm[SL::WY + ty]);
-    }
+    const bool next = kxs[2 * tx + 1] != kxs[2 * tx];
+    const float2 WXv = make_float2(sm[SL::WX + 2 * tx], sm[SL::WX + 2 * tx + 1]);
+    const float2 WYv = bc2(sm[SL::WY + ty]);
 
     // cooperative copy of a node plane's tile
     int csrc[GCOPY];
@@ -198,29 +193,22 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
                 nu[e] = fmaf(t, nu[e + GTP], nu[e]);
         }
     };
-    // displacement plane K of the pair: the value at the first column's first node (U) and the
-    // bilinear interpolation of the in-plane differences to it (B)
-    auto column_pair = [&](int K, float U[3], float2 B[3]) {
-        const float *nu = sm + SL::N + (K % GSLOT_N) * 2 * GTP + lky * GTX + lkx;
-#pragma unroll
-        for (int c = 0; c < 3; c++) {
-            const float *p = nu + c * (GTY * GTX);
-            const float u00 = p[0], u10 = p[1], u20 = p[2];
-            const float u01 = p[GTX], u11 = p[GTX + 1], u21 = p[GTX + 2];
-            const float dy = u01 - u00;
-            U[c] = u00;
-            const float2 X = fma2(C1, bc2(u10 - u00), mul2(C2, bc2(u20 - u10)));
-            const float2 Y = fma2(C1, bc2(u11 - u01), fma2(C2, bc2(u21 - u11), bc2(dy)));
-            B[c] = lerp2(X, Y, WYv);
-        }
+    // values of component c of a row of node plane K at the first and second node of either column
+    auto node_row = [&](const float *p, float2 &a, float2 &b) {
+        const float u0 = p[0], u1 = p[1], u2 = p[2];
+        a = make_float2(u0, next ? u1 : u0);
+        b = make_float2(u1, next ? u2 : u1);
     };
     auto zclamp = [&](int z) { return min(max(z, 0), mz - 1); };
 
     int Kcur = -1;                 // node interval of the plane issued last
     int pend = -1;                 // node plane copied in, its trial values still to form
-    float2 Bl[3], Dd[3];           // in-plane part at the interval's lower plane, and at the upper relative to U
-    float rem[3];                  // U less its whole voxels
-    int bx0 = 0, bx1 = 0, by = 0, bz = 0;
+    // Per column, of the interval: the in-plane interpolation of the node differences to the
+    // value at the first node, on the lower and the upper node plane, and that value less its
+    // whole voxels (rem) - the operations of sample_coord and grid_convert_point, in their order,
+    // so that a sample next to a cell face falls into the same cell in either implementation
+    float2 Bl[3], Dd[3], rem[3];
+    int cb[2][3] = {};             // integer bases of the sample cells (with MAGI taken off; z: + the plane)
     bool ok0 = true, ok1 = true;
     float2 pc[8], fr[3];
     float4 bn0 = make_float4(0.f, 0.f, 0.f, 0.f), bn1 = bn0;
@@ -249,33 +237,40 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
         wq = __ldg(g.pw1[2] + zn);
         if (K != Kcur) {   // uniform over the CTA
             Kcur = K;
-            float Ulo[3], Uhi[3];
-            float2 Bhi[3];
-            column_pair(K, Ulo, Bl);
-            column_pair(K + 1, Uhi, Bhi);
-            float q0max = 0.f;
-            float2 acc = make_float2(0.f, 0.f);
-            int qb[3];
+            const float *nl = sm + SL::N + (K % GSLOT_N) * 2 * GTP + lky * GTX + lkx;
+            const float *nh = sm + SL::N + ((K + 1) % GSLOT_N) * 2 * GTP + lky * GTX + lkx;
+            float2 q0max = make_float2(0.f, 0.f), acc = q0max;
 #pragma unroll
             for (int c = 0; c < 3; c++) {
+                const int o = c * (GTY * GTX);
+                float2 u0, d100, d010, d110, d001, d101, d011, d111;
+                node_row(nl + o, u0, d100);
+                node_row(nl + o + GTX, d010, d110);
+                node_row(nh + o, d001, d101);
+                node_row(nh + o + GTX, d011, d111);
+                d100 = sub2(d100, u0);
+                d010 = sub2(d010, u0);
+                d110 = sub2(d110, u0);
+                d001 = sub2(d001, u0);
+                d101 = sub2(d101, u0);
+                d011 = sub2(d011, u0);
+                d111 = sub2(d111, u0);
+                Bl[c] = lerp2(mul2(WXv, d100), lerp2(d010, d110, WXv), WYv);
+                Dd[c] = lerp2(lerp2(d001, d101, WXv), lerp2(d011, d111, WXv), WYv);
                 const float ih = g.ih[c];
-                const float q0 = Ulo[c] * ih;
-                const float qi = floorf(q0);
-                rem[c] = fmaf(-qi, g.h[c], Ulo[c]);   // |rem| <~ h
-                q0max = fmaxf(q0max, fabsf(q0));
-                qb[c] = (int)qi;
-                const float du = Uhi[c] - Ulo[c];
-                Dd[c] = make_float2(du + Bhi[c].x, du + Bhi[c].y);
+                const float2 q0 = mul2(u0, bc2(ih));
+                const float2 qi = make_float2(floorf(q0.x), floorf(q0.y));
+                rem[c] = make_float2(fmaf(-qi.x, g.h[c], u0.x), fmaf(-qi.y, g.h[c], u0.y));   // |rem| <~ h
+                q0max = make_float2(fmaxf(q0max.x, fabsf(q0.x)), fmaxf(q0max.y, fabsf(q0.y)));
+                const int base = (c == 0 ? xa : c == 1 ? y : 0) + 2 - MAGI;
+                cb[0][c] = (int)qi.x + base;
+                cb[1][c] = (int)qi.y + base + (c == 0 ? 1 : 0);
                 const float2 b = mul2(Bl[c], bc2(ih)), d = mul2(Dd[c], bc2(ih));
                 acc = fma2(b, b, fma2(d, d, acc));
             }
             // the displacement of every plane between them is below 1e6 voxels and finite
-            ok0 = q0max < 1.0e6f && acc.x < 1.0e12f;
-            ok1 = q0max < 1.0e6f && acc.y < 1.0e12f;
-            bx0 = qb[0] + xa + 2 - MAGI;
-            bx1 = bx0 + 1;
-            by = qb[1] + y + 2 - MAGI;
-            bz = qb[2] + 2 - MAGI;
+            ok0 = q0max.x < 1.0e6f && acc.x < 1.0e12f;
+            ok1 = q0max.y < 1.0e6f && acc.y < 1.0e12f;
             if (!first) {   // plane K - 1's slot
                 issue_plane(K + 2);
                 pend = K + 2;
@@ -287,7 +282,7 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
         int ix[2][3];
 #pragma unroll
         for (int c = 0; c < 3; c++) {
-            const float2 f = mul2(add2(bc2(rem[c]), lerp2(Bl[c], Dd[c], WZ)), bc2(g.ih[c]));
+            const float2 f = mul2(add2(rem[c], lerp2(Bl[c], Dd[c], WZ)), bc2(g.ih[c]));
             const float2 fm = __fadd2_rd(f, bc2(MAGF));
             fr[c] = sub2(f, sub2(fm, bc2(MAGF)));
             ix[0][c] = __float_as_int(fm.x);
@@ -296,8 +291,9 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
 #pragma unroll
         for (int k = 0; k < 2; k++) {
             float v[8];
-            corners_padded(static_cast<const TemplateElem<float>::type *>(a.T), ix[k][0] + (k ? bx1 : bx0), ix[k][1] + by, ix[k][2] + bz + z1, k ? ok1 : ok0, CXM, CYM,
-                           CZM, MXP, MYP, SXYP, v);
+            corners_padded(static_cast<const TemplateElem<float>::type *>(a.T), ix[k][0] + cb[k][0],
+                           ix[k][1] + cb[k][1], ix[k][2] + cb[k][2] + z1, k ? ok1 : ok0, CXM, CYM, CZM, MXP, MYP, SXYP,
+                           v);
 #pragma unroll
             for (int j = 0; j < 8; j++) {
                 if (k)
