@@ -480,7 +480,8 @@ int reg_set_images(reg_handle c, const float *R, const float *T, const int dims[
     const long long nv0 = c->L[0].nv;
     c->have_images = false;
 
-    // finest images, then the pyramid: R on the handle's stream, T on the side stream
+    // finest images, the pyramid and the fused passes' copies (BF16 rounded to nearest
+    // even): R and its field on the handle's stream, T on the side stream
     cudaMemcpyKind kind = ptr_is_device ? cudaMemcpyDeviceToDevice : cudaMemcpyHostToDevice;
     CK(cudaEventRecord(c->ev_side, c->stream));
     CK(cudaStreamWaitEvent(c->side, c->ev_side, 0));
@@ -491,16 +492,14 @@ int reg_set_images(reg_handle c, const float *R, const float *T, const int dims[
         CK(launch_restrict(c->L[l - 1].T, c->L[l - 1].m, c->L[l].T, c->side));
         c->launches += 2;
     }
-    CK(cudaEventRecord(c->ev_side, c->side));
-    CK(cudaStreamWaitEvent(c->stream, c->ev_side, 0));
-    for (int l = 0; l < c->levels; l++) {   // the fused pass's copies; BF16 rounded to nearest even
+    for (int l = 0; l < c->levels; l++) {
         if (c->L[l].Rb) {
             CK(launch_to_bf16(c->L[l].R, c->L[l].Rb, c->L[l].nv, c->stream));
-            CK(launch_pad_template(c->L[l].T, c->L[l].m, c->L[l].Tb, c->stream));
+            CK(launch_pad_template(c->L[l].T, c->L[l].m, c->L[l].Tb, c->side));
             c->launches += 2;
         }
         if (c->L[l].Tp) {
-            CK(launch_pad_template(c->L[l].T, c->L[l].m, c->L[l].Tp, c->stream));
+            CK(launch_pad_template(c->L[l].T, c->L[l].m, c->L[l].Tp, c->side));
             c->launches += 1;
         }
         if (c->L[l].Rn) {
@@ -508,6 +507,8 @@ int reg_set_images(reg_handle c, const float *R, const float *T, const int dims[
             c->launches += 1;
         }
     }
+    CK(cudaEventRecord(c->ev_side, c->side));
+    CK(cudaStreamWaitEvent(c->stream, c->ev_side, 0));
     // tiling of the fused pass per level: forced, autotuned (at u = 0, with the
     // direction buffer as the zero field) or the default rule
     for (int l = 0; l < c->levels; l++) {
