@@ -11,6 +11,8 @@ this package marshals arguments and uses PyTorch only for device memory and
 streams.  Arrays: images (m_z, m_y, m_x) float32; displacements
 (3, n_z, n_y, n_x) float32 in mm (component planes x, y, z).
 """
+import math
+
 import numpy as np
 import torch
 
@@ -78,6 +80,7 @@ class Registration:
         self.stream = stream if stream is not None else torch.cuda.current_stream()
         self.h = _lib.reg_create(self.cfg, self.stream.cuda_stream)
         self.dims = None
+        self._shapes = {}   # node_shape per level, until the next images
 
     # -- images -------------------------------------------------------------
     def set_images(self, R, T, spacing):
@@ -98,6 +101,7 @@ class Registration:
             raise ValueError("R and T must be 3D arrays of equal shape")
         mz, my, mx = R.shape
         self.dims = (mx, my, mz)
+        self._shapes = {}
         _lib.reg_set_images(self.h, pr, pt, self.dims, spacing, dev)
         self._keep = (R, T)  # device copies are taken on the handle's stream
         return self
@@ -115,8 +119,11 @@ class Registration:
         return _lib.reg_level_split(self.h, level)
 
     def node_shape(self, level=0):
-        n = self.level_info(level)["nodes"]
-        return (3, n[2], n[1], n[0])
+        shape = self._shapes.get(level)
+        if shape is None:
+            n = self.level_info(level)["nodes"]
+            shape = self._shapes[level] = (3, n[2], n[1], n[0])
+        return shape
 
     def level_image(self, level, which="R"):
         m = self.level_info(level)["dims"]
@@ -177,7 +184,7 @@ class Registration:
         shape = self.node_shape(level)
         if not (isinstance(u, torch.Tensor) and u.is_cuda and u.dtype == torch.float32):
             raise TypeError("u must be a float32 CUDA tensor")
-        if tuple(u.shape) != shape and u.numel() != int(np.prod(shape)):
+        if tuple(u.shape) != shape and u.numel() != math.prod(shape):
             raise ValueError("u has %s elements, level %d needs %s" % (tuple(u.shape), level, shape))
         return u.contiguous()
 
@@ -202,7 +209,7 @@ class RegObjective(torch.autograd.Function):
     def forward(ctx, u, reg, level=0):
         J, D, S, grad = reg.eval(u.detach(), level)
         ctx.save_for_backward(grad)
-        return torch.tensor(J, dtype=torch.float64, device=u.device)
+        return torch.full((), J, dtype=torch.float64, device=u.device)   # a fill, not a blocking transfer
 
     @staticmethod
     def backward(ctx, gJ):

@@ -97,6 +97,7 @@ struct EvalScratch {
     double *partials = nullptr;   // block partial sums
     int max_partials = 0;
     double *scal = nullptr;       // [J, D, S] on the device
+    double *scal_host = nullptr;  // [J, D, S] in page-locked host memory the device writes
     size_t part_floats = 0;
 };
 
@@ -113,7 +114,7 @@ struct LbfgsBuffers {
     int cnt_len = 0;
     unsigned *gbar = nullptr;           // [arrivals, generation, flags] of the whole-level kernel's grid barrier
     LbfgsState *st = nullptr;           // device
-    LbfgsState *st_host = nullptr;      // pinned mirror
+    LbfgsState *st_host = nullptr;      // pinned mirror (EvalScratch::scal_host lies behind it)
     double *scal_t = nullptr;           // [J, D, S] of the trial point
 };
 
@@ -137,6 +138,7 @@ struct reg_ctx {
     EvalScratch es;
     LbfgsBuffers lb;
     std::string err;
+    void *arena = nullptr;    // every device buffer of the geometry
     // CUDA graph of one L-BFGS iteration per level (built lazily)
     cudaGraphExec_t iter_graph[REG_MAX_LEVELS] = {};
     cudaGraphExec_t init_graph[REG_MAX_LEVELS] = {};

@@ -165,11 +165,14 @@ cudaError_t launch_eval(reg_ctx *c, int level, const float *ub, const float *dir
     // wave: fork before, join before the gradient assembly.  Captured, the two
     // become parallel graph branches.  With the batched form's arithmetic the
     // fused pass forms it itself, with one S partial per tile.
-    e = cudaEventRecord(c->ev_fork, s);
-    if (e == cudaSuccess)
-        e = cudaStreamWaitEvent(c->side, c->ev_fork, 0);
-    if (e != cudaSuccess)
-        return e;
+    e = cudaSuccess;
+    if (!curv_in_pass) {
+        e = cudaEventRecord(c->ev_fork, s);
+        if (e == cudaSuccess)
+            e = cudaStreamWaitEvent(c->side, c->ev_fork, 0);
+        if (e != cudaSuccess)
+            return e;
+    }
     if (c->time_ngf)
         e = cudaEventRecord(c->kev[0], s);
     if (e == cudaSuccess) {
@@ -194,11 +197,11 @@ cudaError_t launch_eval(reg_ctx *c, int level, const float *ub, const float *dir
             : k_curv_w<false><<<gw, CURV_NODES, 0, c->side>>>(g, ub, dir, t_dev, c->es.w, pS, planes);
         c->launches += 1;
         e = cudaGetLastError();
+        if (e == cudaSuccess)
+            e = cudaEventRecord(c->ev_join, c->side);
+        if (e == cudaSuccess)
+            e = cudaStreamWaitEvent(s, c->ev_join, 0);
     }
-    if (e == cudaSuccess)
-        e = cudaEventRecord(c->ev_join, c->side);
-    if (e == cudaSuccess)
-        e = cudaStreamWaitEvent(s, c->ev_join, 0);
     if (e != cudaSuccess)
         return e;
     double hy = L.H[0] * L.H[1] * L.H[2];

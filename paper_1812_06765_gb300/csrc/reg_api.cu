@@ -13,59 +13,20 @@ namespace {
 
 thread_local std::string g_create_err;
 
-void free_level(Level &L)
-{
-    cudaFree(L.R);
-    cudaFree(L.T);
-    cudaFree(L.Tp);
-    cudaFree(L.Rn);
-    cudaFree(L.Rb);
-    cudaFree(L.Tb);
-    for (int d = 0; d < 3; d++) {
-        cudaFree(L.pk0[d]);
-        cudaFree(L.pw1[d]);
-        cudaFree(L.tfirst[d]);
-        cudaFree(L.tcnt[d]);
-        cudaFree(L.tw[d]);
-        cudaFree(L.qk0[d]);
-        cudaFree(L.qw1[d]);
-    }
-    L = Level();
-}
-
+// Every device buffer of a geometry lies in one allocation (allocate_buffers)
 void free_buffers(reg_ctx *c)
 {
     for (int l = 0; l < REG_MAX_LEVELS; l++) {
-        free_level(c->L[l]);
+        c->L[l] = Level();
         if (c->iter_graph[l]) cudaGraphExecDestroy(c->iter_graph[l]);
         if (c->init_graph[l]) cudaGraphExecDestroy(c->init_graph[l]);
         c->iter_graph[l] = nullptr;
         c->init_graph[l] = nullptr;
     }
-    EvalScratch &e = c->es;
-    cudaFree(e.Tw);
-    cudaFree(e.dT);
-    cudaFree(e.v);
-    cudaFree(e.r);
-    cudaFree(e.w);
-    cudaFree(e.part);
-    cudaFree(e.partials);
-    cudaFree(e.scal);
+    cudaFree(c->arena);
+    c->arena = nullptr;
     c->es = EvalScratch();
-    LbfgsBuffers &b = c->lb;
-    cudaFree(b.u);
-    cudaFree(b.pdir);
-    cudaFree(b.g);
-    cudaFree(b.gt);
-    cudaFree(b.P);
-    cudaFree(b.Y);
-    cudaFree(b.partials);
-    cudaFree(b.gpart);
-    cudaFree(b.gbar);
-    cudaFree(b.cnt);
-    cudaFree(b.st);
-    cudaFree(b.scal_t);
-    if (b.st_host) cudaFreeHost(b.st_host);
+    if (c->lb.st_host) cudaFreeHost(c->lb.st_host);
     c->lb = LbfgsBuffers();
     c->have_images = false;
 }
@@ -122,15 +83,6 @@ int validate_config(const reg_config *cfg, std::string &msg)
     return REG_ERR_ARG;
 }
 
-template <typename T>
-cudaError_t upload(T **dst, const std::vector<T> &src)
-{
-    cudaError_t e = cudaMalloc((void **)dst, sizeof(T) * (src.empty() ? 1 : src.size()));
-    if (e != cudaSuccess) return e;
-    if (src.empty()) return cudaSuccess;
-    return cudaMemcpy(*dst, src.data(), sizeof(T) * src.size(), cudaMemcpyHostToDevice);
-}
-
 // Per-dimension tables of P (voxel i -> node k0, weight of k0 + 1) and of P^T
 // (node k -> first voxel, count, weights), from the hat functions at voxel
 // centres t = (i + 1/2) h / H (Sec. 2.2, Eq. 3: weights and index sets are
@@ -158,14 +110,17 @@ AxisTables axis_tables(int m, double h, double H, int n)
     a.first.assign(n, 0);
     a.cnt.assign(n, 0);
     std::vector<std::vector<double>> ws(n);
-    for (int k = 0; k < n; k++) {
-        for (int i = 0; i < m; i++) {
-            double w = 1.0 - fabs(t[i] - k);
+    for (int i = 0; i < m; i++) {
+        const int kf = (int)floor(t[i]);   // the hats of kf and kf + 1 reach the voxel
+        for (int k = kf < 0 ? 0 : kf; k <= kf + 1 && k < n; k++) {
+            const double w = 1.0 - fabs(t[i] - k);
             if (w > 0.0) {
                 if (ws[k].empty()) a.first[k] = i;
                 ws[k].push_back(w);
             }
         }
+    }
+    for (int k = 0; k < n; k++) {
         a.cnt[k] = (int)ws[k].size();
         if (a.cnt[k] > a.maxw) a.maxw = a.cnt[k];
     }
@@ -175,24 +130,50 @@ AxisTables axis_tables(int m, double h, double H, int n)
     return a;
 }
 
-cudaError_t build_tables(Level &L)
+// Lays buffers out one after another, each at a 256-byte boundary: first with
+// no base, to learn the size, then into the allocation of that size.
+struct Carver {
+    char *base = nullptr;
+    size_t used = 0;
+    template <typename T>
+    void take(T *&p, size_t count)
+    {
+        used = (used + 255) & ~(size_t)255;
+        p = base ? reinterpret_cast<T *>(base + used) : nullptr;
+        used += sizeof(T) * (count > 0 ? count : 1);
+    }
+};
+
+// The tables of a handle: carved from the head of its allocation and, at the
+// same offsets, from a host copy that goes up in one transfer.
+struct TableCarver {
+    Carver dev, host;
+    template <typename T>
+    void put(T *&p, const std::vector<T> &src)
+    {
+        T *h = nullptr;
+        dev.take(p, src.size());
+        host.take(h, src.size());
+        if (h && !src.empty())
+            memcpy(h, src.data(), sizeof(T) * src.size());
+    }
+};
+
+void carve_tables(Level &L, const AxisTables a[3], TableCarver &tc)
 {
     for (int d = 0; d < 3; d++) {
-        const AxisTables a = axis_tables(L.m[d], L.h[d], L.H[d], L.n[d]);
-        L.tmaxw[d] = a.maxw;
-        cudaError_t e;
-        if ((e = upload(&L.pk0[d], a.k0)) != cudaSuccess) return e;
-        if ((e = upload(&L.pw1[d], a.w1)) != cudaSuccess) return e;
-        if ((e = upload(&L.tfirst[d], a.first)) != cudaSuccess) return e;
-        if ((e = upload(&L.tcnt[d], a.cnt)) != cudaSuccess) return e;
-        if ((e = upload(&L.tw[d], a.tw)) != cudaSuccess) return e;
+        L.tmaxw[d] = a[d].maxw;
+        tc.put(L.pk0[d], a[d].k0);
+        tc.put(L.pw1[d], a[d].w1);
+        tc.put(L.tfirst[d], a[d].first);
+        tc.put(L.tcnt[d], a[d].cnt);
+        tc.put(L.tw[d], a[d].tw);
     }
-    return cudaSuccess;
 }
 
 // Prolongation tables of a fine level from the next coarser one: fine node j
 // at j H_f in mm, coarse coordinate j H_f / H_c.
-cudaError_t build_prolong_tables(Level &F, const Level &C)
+void carve_prolong_tables(Level &F, const Level &C, TableCarver &tc)
 {
     for (int d = 0; d < 3; d++) {
         std::vector<int> k0(F.n[d]);
@@ -205,11 +186,9 @@ cudaError_t build_prolong_tables(Level &F, const Level &C)
             k0[j] = k;
             w1[j] = (float)(t - k);
         }
-        cudaError_t e;
-        if ((e = upload(&F.qk0[d], k0)) != cudaSuccess) return e;
-        if ((e = upload(&F.qw1[d], w1)) != cudaSuccess) return e;
+        tc.put(F.qk0[d], k0);
+        tc.put(F.qw1[d], w1);
     }
-    return cudaSuccess;
 }
 
 }  // namespace
@@ -256,90 +235,116 @@ int cuda_err(reg_ctx *c, cudaError_t e, const char *what)
 }
 
 // Device buffers of a new image geometry: level images and tables, evaluation
-// scratch and the L-BFGS vectors (all sized by the finest level).
+// scratch and the L-BFGS vectors (all sized by the finest level).  One
+// allocation and one upload of tables for all of them: a handle made for one
+// registration of 64^3 spent 1.5 ms of 2.55 on about 45 allocations, 42 small
+// transfers and their release.
 int allocate_buffers(reg_ctx *c)
 {
     const reg_config &cfg = c->cfg;
-    long long nmax = 0;
+    long long nmax = 0, mp_vox = 0;   // mp_vox: largest level served by the multi-pass kernels
     int maxpart = 0;
+    size_t part = 0;                  // largest tile-partial buffer of the fused passes
+    std::vector<AxisTables> axes(3 * c->levels);
     for (int l = 0; l < c->levels; l++) {
         Level &L = c->L[l];
-        CK(cudaMalloc(&L.R, sizeof(float) * L.nv));
-        CK(cudaMalloc(&L.T, sizeof(float) * L.nv));
-        CK(build_tables(L));
-        if (l > 0) CK(build_prolong_tables(c->L[l - 1], L));
+        for (int d = 0; d < 3; d++)
+            axes[3 * l + d] = axis_tables(L.m[d], L.h[d], L.H[d], L.n[d]);
         if (3 * L.nn > nmax) nmax = 3 * L.nn;
-        int p = eval_partials_needed(L);
+        const int p = eval_partials_needed(L);
         if (p > maxpart) maxpart = p;
+        size_t f = 0;
+        if (use_fused(c, l)) {
+            f = fused_part_floats(L, c->num_sms);
+        } else if (use_general(c, l)) {
+            L.gen_split = general_split(L.m, c->num_sms);
+            f = general_part_floats(L);
+        } else if (L.nv > mp_vox) {
+            mp_vox = L.nv;
+        }
+        if (f > part) part = f;
     }
     EvalScratch &es = c->es;
-    long long mp_vox = 0;      // largest level served by the multi-pass kernels
-    size_t part = 0;           // largest tile-partial buffer of the fused pass
-    for (int l = 0; l < c->levels; l++) {
-        if (use_fused(c, l)) {
-            size_t p = fused_part_floats(c->L[l], c->num_sms);
-            if (p > part) part = p;
-        } else if (use_general(c, l)) {
-            c->L[l].gen_split = general_split(c->L[l].m, c->num_sms);
-            size_t p = general_part_floats(c->L[l]);
-            if (p > part) part = p;
-        } else if (c->L[l].nv > mp_vox) {
-            mp_vox = c->L[l].nv;
-        }
-    }
-    if (mp_vox > 0) {
-        CK(cudaMalloc(&es.Tw, sizeof(float) * mp_vox));
-        CK(cudaMalloc(&es.dT, sizeof(float) * 3 * mp_vox));
-        CK(cudaMalloc(&es.v, sizeof(float) * 3 * mp_vox));
-        CK(cudaMalloc(&es.r, sizeof(float) * 3 * mp_vox));
-    }
-    if (part > 0) {
-        CK(cudaMalloc(&es.part, sizeof(float) * part));
-        es.part_floats = part;
-    }
-    // the fused passes read T through a zero-bordered copy (FP32, or BF16 beside a BF16 R)
-    for (int l = 0; l < c->levels; l++)
-        if (use_fused(c, l) || use_general(c, l)) {
-            const long long np = padded_voxels(c->L[l].m);
-            if (cfg.image_dtype == 1 && use_fused(c, l)) {
-                CK(cudaMalloc(&c->L[l].Rb, sizeof(__nv_bfloat16) * c->L[l].nv));
-                CK(cudaMalloc(&c->L[l].Tb, sizeof(__nv_bfloat162) * np));
-            } else {
-                CK(cudaMalloc(&c->L[l].Tp, sizeof(float) * np));
-            }
-            CK(cudaMalloc(&c->L[l].Rn, sizeof(float4) * rn_voxels(c->L[l].m)));
-        }
-    CK(cudaMalloc(&es.w, sizeof(float) * nmax));
-    CK(cudaMalloc(&es.partials, sizeof(double) * maxpart));
-    CK(cudaMalloc(&es.scal, sizeof(double) * 4));
-    es.max_partials = maxpart;
     LbfgsBuffers &b = c->lb;
+    es.part_floats = part;
+    es.max_partials = maxpart;
     b.n = nmax;
     b.slots = cfg.lbfgs_mem + 1;
-    CK(cudaMalloc(&b.u, sizeof(float) * nmax));
-    CK(cudaMalloc(&b.pdir, sizeof(float) * nmax));
-    CK(cudaMalloc(&b.g, sizeof(float) * nmax));
-    CK(cudaMalloc(&b.gt, sizeof(float) * nmax));
-    const long long nring = (nmax + 3) & ~3LL;   // slot stride rounded up to 16 bytes
-    CK(cudaMalloc(&b.P, sizeof(float) * nring * b.slots));
-    CK(cudaMalloc(&b.Y, sizeof(float) * nring * b.slots));
     // the largest per-block layout is that of reg_lbfgs_direction's pair dots
     b.max_partials = 4 * c->num_sms * (2 + 2 * LB_MAXM + 2 * LB_MAXM * LB_MAXM) + 1024;
-    CK(cudaMalloc(&b.partials, sizeof(float) * b.max_partials));
-    {   // group sums and arrival counters of the vector passes (<= 4 blocks per SM)
-        const int groups = (4 * c->num_sms + LB_RG - 1) / LB_RG;
-        CK(cudaMalloc(&b.gpart, sizeof(float2) * groups * (2 + 4 * LB_MAXS)));
-        b.cnt_len = groups + 1;
-        // one more counter past them: reg_lbfgs_direction's
-        CK(cudaMalloc(&b.cnt, sizeof(unsigned) * (b.cnt_len + 1)));
-        CK(cudaMemset(b.cnt, 0, sizeof(unsigned) * (b.cnt_len + 1)));
-        CK(cudaMalloc(&b.gbar, 3 * sizeof(unsigned)));
-        CK(cudaMemset(b.gbar, 0, 3 * sizeof(unsigned)));
-    }
-    CK(cudaMalloc(&b.st, sizeof(LbfgsState)));
-    CK(cudaMalloc(&b.scal_t, sizeof(double) * 4));
-    CK(cudaMallocHost(&b.st_host, sizeof(LbfgsState)));
-    CK(cudaMemsetAsync(b.st, 0, sizeof(LbfgsState), c->stream));
+    // group sums and arrival counters of the vector passes (<= 4 blocks per SM)
+    const int groups = (4 * c->num_sms + LB_RG - 1) / LB_RG;
+    b.cnt_len = groups + 1;
+    const long long nring = (nmax + 3) & ~3LL;   // slot stride rounded up to 16 bytes
+    size_t table_bytes = 0, zero_begin = 0, zero_end = 0;
+    std::vector<char> table_host;
+    auto carve = [&](Carver &m) {
+        TableCarver tc;
+        tc.dev.base = m.base;
+        tc.host.base = m.base ? table_host.data() : nullptr;
+        for (int l = 0; l < c->levels; l++) {
+            carve_tables(c->L[l], &axes[3 * l], tc);
+            if (l > 0) carve_prolong_tables(c->L[l - 1], c->L[l], tc);
+        }
+        m.used = table_bytes = tc.dev.used;
+        // zeroed: arrival counters (one more past the vector passes': reg_lbfgs_direction's),
+        // the whole-level kernel's barrier, the solver state
+        char *mark = nullptr;
+        m.take(mark, 1);
+        zero_begin = m.used - 1;
+        m.take(b.cnt, b.cnt_len + 1);
+        m.take(b.gbar, 3);
+        m.take(b.st, 1);
+        zero_end = m.used;
+        for (int l = 0; l < c->levels; l++) {
+            Level &L = c->L[l];
+            m.take(L.R, L.nv);
+            m.take(L.T, L.nv);
+            // the fused passes read T through a zero-bordered copy (FP32, or BF16 beside a BF16 R)
+            if (use_fused(c, l) || use_general(c, l)) {
+                if (cfg.image_dtype == 1 && use_fused(c, l)) {
+                    m.take(L.Rb, L.nv);
+                    m.take(L.Tb, padded_voxels(L.m));
+                } else {
+                    m.take(L.Tp, padded_voxels(L.m));
+                }
+                m.take(L.Rn, rn_voxels(L.m));
+            }
+        }
+        if (mp_vox > 0) {
+            m.take(es.Tw, mp_vox);
+            m.take(es.dT, 3 * mp_vox);
+            m.take(es.v, 3 * mp_vox);
+            m.take(es.r, 3 * mp_vox);
+        }
+        if (part > 0) m.take(es.part, part);
+        m.take(es.w, nmax);
+        m.take(es.partials, maxpart);
+        m.take(es.scal, 4);
+        m.take(b.u, nmax);
+        m.take(b.pdir, nmax);
+        m.take(b.g, nmax);
+        m.take(b.gt, nmax);
+        m.take(b.P, nring * b.slots);
+        m.take(b.Y, nring * b.slots);
+        m.take(b.partials, b.max_partials);
+        m.take(b.gpart, (size_t)groups * (2 + 4 * LB_MAXS));
+        m.take(b.scal_t, 4);
+    };
+    Carver size;
+    carve(size);
+    CK(cudaMalloc(&c->arena, size.used));
+    table_host.assign(table_bytes, 0);
+    Carver at;
+    at.base = static_cast<char *>(c->arena);
+    carve(at);
+    CK(cudaMemcpy(c->arena, table_host.data(), table_bytes, cudaMemcpyHostToDevice));
+    CK(cudaMemsetAsync(at.base + zero_begin, 0, zero_end - zero_begin, c->stream));
+    // page-locked, readable and writable from the device: the state's mirror and an evaluation's [J, D, S]
+    void *host = nullptr;
+    CK(cudaMallocHost(&host, sizeof(LbfgsState) + 4 * sizeof(double)));
+    b.st_host = static_cast<LbfgsState *>(host);
+    es.scal_host = reinterpret_cast<double *>(b.st_host + 1);
     return REG_OK;
 }
 
@@ -656,14 +661,13 @@ int reg_eval_objective_grad(reg_handle c, int level, const float *u_dev, float *
         return set_err(c, REG_ERR_ARG, "reg_eval_objective_grad: level %d out of range", level);
     if (!u_dev || !grad_dev) return set_err(c, REG_ERR_ARG, "reg_eval_objective_grad: NULL vector");
     c->time_ngf = true;
-    cudaError_t le = launch_eval(c, level, u_dev, nullptr, nullptr, grad_dev, c->es.scal, -1, c->stream);
+    cudaError_t le = launch_eval(c, level, u_dev, nullptr, nullptr, grad_dev, c->es.scal_host, -1, c->stream);
     c->time_ngf = false;
     c->kev_valid = le == cudaSuccess;
     CK(le);
     if (J || D || S) {
-        double h[3];
-        CK(cudaMemcpyAsync(h, c->es.scal, sizeof h, cudaMemcpyDeviceToHost, c->stream));
-        CK(cudaStreamSynchronize(c->stream));
+        CK(cudaStreamSynchronize(c->stream));   // the final reduction has written them to host memory
+        const double h[3] = {c->es.scal_host[0], c->es.scal_host[1], c->es.scal_host[2]};
         if (J) *J = h[0];
         if (D) *D = h[1];
         if (S) *S = h[2];
