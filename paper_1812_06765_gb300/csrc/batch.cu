@@ -85,6 +85,7 @@ struct BatchDev {
     PairLevel *pl = nullptr;
     int *off = nullptr;      // [3][npairs + 1]: tiles, gather blocks, vector blocks
     int *counters = nullptr; // [4]: runs of the iteration and search conditions, then their last values
+    int *searching() const { return counters + 4; }   // [npairs]: pairs the current evaluation covers
 };
 
 struct CaptureGuard {
@@ -135,12 +136,11 @@ struct BatchLaunch {
 
     cudaError_t eval(int mode, cudaStream_t s) const
     {
-        // the fused pass also forms each pair's curvature Laplacian and S partials
-        cudaError_t e = launch_fused_batch(d->pl, d->off, npairs, tiles, mode, bf16, g_fused, device, s);
+        // the fused pass also forms each pair's curvature Laplacian and S partials; the gather
+        // reduces J, D, S and (mode 1) takes the line-search decisions
+        cudaError_t e = launch_fused_batch(d->pl, d->off, npairs, tiles, d->searching(), mode, bf16, g_fused, device, s);
         if (e == cudaSuccess)
-            e = launch_gather_batch(d->pl, d->off + (npairs + 1), npairs, nodes, mode, g_nodes, s);
-        if (e == cudaSuccess)
-            e = launch_finalize_batch(d->pl, npairs, mode, s);
+            e = launch_gather_batch(d->pl, d->off + (npairs + 1), npairs, nodes, d->searching(), mode, g_nodes, s);
         return e;
     }
     cudaError_t vec(int step, cudaStream_t s) const
@@ -164,7 +164,7 @@ struct BatchLaunch {
     } while (0)
 
 // The whole level for all pairs: init, then WHILE any pair iterates
-// { direction; WHILE any pair searches { objective at the trial points; Armijo }; accept }.
+// { direction; WHILE any pair searches { objective at the trial points with Armijo }; accept }.
 cudaError_t build_batch_graph(const BatchLaunch &B, cudaStream_t cs, cudaGraphExec_t *out)
 {
     cudaGraph_t G = nullptr;
@@ -209,7 +209,6 @@ cudaError_t build_batch_graph(const BatchLaunch &B, cudaStream_t cs, cudaGraphEx
         BK(cudaStreamBeginCaptureToGraph(cs, ls_body, nullptr, nullptr, 0, mode));
         guard.active = true;
         BK(B.eval(1, cs));
-        BK(B.ctl(LB_ARMIJO, cs));
         BK(B.cond(1, h_ls, cs));
         guard.active = false;
         BK(cudaStreamEndCapture(cs, &g2));
@@ -294,7 +293,8 @@ int batch_tiling_rule(reg_handle *hs, int n, int l, const std::vector<FusedSplit
             if (r >= 0)
                 e = cudaEventRecord(e0, s);
             if (e == cudaSuccess)
-                e = launch_fused_batch(d.pl, d.off, n, tiles, 0, bf16, cap(tiles, (long long)fused_slots(c0->num_sms)), c0->device, s);
+                e = launch_fused_batch(d.pl, d.off, n, tiles, d.searching(), 0, bf16,
+                                       cap(tiles, (long long)fused_slots(c0->num_sms)), c0->device, s);
             if (e == cudaSuccess && r >= 0)
                 e = cudaEventRecord(e1, s);
             if (e == cudaSuccess && r >= 0)
@@ -356,7 +356,6 @@ cudaError_t run_batch_level_host(const BatchLaunch &B, int *counters, cudaStream
         HK(cond(1, ls));
         while (ls && rounds++ < max_rounds) {
             HK(B.eval(1, s));
-            HK(B.ctl(LB_ARMIJO, s));
             HK(cond(1, ls));
         }
         HK(B.vec(3, s));
@@ -407,7 +406,7 @@ extern "C" int reg_register_batch(reg_handle *hs, int n, float **u_out, int out_
     BatchDev d;
     CK(cudaMallocAsync((void **)&d.pl, sizeof(PairLevel) * n, s));
     CK(cudaMallocAsync((void **)&d.off, sizeof(int) * 3 * (n + 1), s));
-    CK(cudaMallocAsync((void **)&d.counters, sizeof(int) * 4, s));
+    CK(cudaMallocAsync((void **)&d.counters, sizeof(int) * (4 + n), s));
     // every pair's own stream work (prolongations, state uploads) is ordered on c0's stream
     for (int i = 0; i < n; i++) {
         CK(cudaMemsetAsync(hs[i]->lb.u, 0, sizeof(float) * 3 * hs[i]->L[start].nn, s));
@@ -510,9 +509,9 @@ extern "C" int reg_register_batch(reg_handle *hs, int n, float **u_out, int out_
         if (e == cudaSuccess)
             e = cudaStreamSynchronize(s);
         CK(e);
-        // launches: init 7; per iteration body 8; per search round 6
+        // launches: init 5; per iteration body 8; per search round 3
         const long long bodies = cnt[0] - 1, rounds = cnt[1] - bodies;
-        launches += 7 + 8 * bodies + 6 * rounds;
+        launches += 5 + 8 * bodies + 3 * rounds;
         for (int i = 0; i < n; i++) {
             reg_ctx *ci = hs[i];
             CK(cudaMemcpyAsync(ci->lb.st_host, ci->lb.st, sizeof(LbfgsState), cudaMemcpyDeviceToHost, s));

@@ -67,12 +67,13 @@ __device__ __forceinline__ int find_pair(const int *__restrict__ off, int npairs
     return lo;
 }
 
-// batched launchers (mode 0: objective at u, 1: at the trial point of pairs still searching)
-cudaError_t launch_fused_batch(const PairLevel *pl, const int *tile_off, int npairs, int total, int mode, bool bf16,
-                               int grid, int device, cudaStream_t s);
-cudaError_t launch_gather_batch(const PairLevel *pl, const int *off, int npairs, int total, int mode, int grid,
-                                cudaStream_t s);
-cudaError_t launch_finalize_batch(const PairLevel *pl, int npairs, int mode, cudaStream_t s);
+// batched launchers (mode 0: objective at u, 1: at the trial point of pairs still searching);
+// the fused pass writes searching[npairs], the gather reads it and ends the evaluation: J, D, S
+// and in mode 1 the line-search decisions
+cudaError_t launch_fused_batch(const PairLevel *pl, const int *tile_off, int npairs, int total, int *searching,
+                               int mode, bool bf16, int grid, int device, cudaStream_t s);
+cudaError_t launch_gather_batch(const PairLevel *pl, const int *off, int npairs, int total, const int *searching,
+                                int mode, int grid, cudaStream_t s);
 // step 0: norms of g, 1: direction, 2: its p0 redo, 3: accept
 cudaError_t launch_lb_vector_batch(const PairLevel *pl, const int *chunk_off, int npairs, int total, int step,
                                    int grid, cudaStream_t s);

@@ -6,7 +6,6 @@
 //   grad_c J += alpha hbar_y L^T w_c     (the symmetric stencil gathered over
 //                                         the zero-extended w)
 // Both passes are node-parallel, one thread per node and all 3 components.
-#include "batch.h"
 #include "internal.h"
 #include "ngf_math.cuh"
 
@@ -121,22 +120,6 @@ __global__ void __launch_bounds__(512) k_finalize(const double *__restrict__ pD,
     finalize_body(pD, nD, pS, nS, hbar_half, alpha, hy_half, scal);
 }
 
-// Batched forms over all pairs of a level.  Mode 0: at u; mode 1: at the trial
-// point, only for pairs still searching.
-__device__ __forceinline__ bool batch_skip(const PairLevel &P, int mode)
-{
-    return mode == 1 && !(P.st->active && P.st->ls_continue);
-}
-
-
-__global__ void __launch_bounds__(512) k_finalize_batch(const PairLevel *__restrict__ pl, int mode)
-{
-    const PairLevel &P = pl[blockIdx.x];
-    if (batch_skip(P, mode))
-        return;
-    finalize_body(P.fa_init.partials, P.nD, P.pS, P.nS, P.hbar_half, P.alpha, P.hy_half, mode ? P.scal_t : P.scal);
-}
-
 }  // namespace
 
 bool is_curv_w_kernel(const void *f)
@@ -144,12 +127,6 @@ bool is_curv_w_kernel(const void *f)
     return f == reinterpret_cast<const void *>(k_curv_w<true>) || f == reinterpret_cast<const void *>(k_curv_w<false>);
 }
 
-
-cudaError_t launch_finalize_batch(const PairLevel *pl, int npairs, int mode, cudaStream_t s)
-{
-    k_finalize_batch<<<npairs, 512, 0, s>>>(pl, mode);
-    return cudaGetLastError();
-}
 
 cudaError_t launch_eval(reg_ctx *c, int level, const float *ub, const float *dir, const double *t_dev, float *grad,
                         double *scal_out, int ctl_phase, cudaStream_t s)

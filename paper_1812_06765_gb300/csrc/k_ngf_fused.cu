@@ -82,16 +82,21 @@ __global__ void __launch_bounds__(BX * BY, CTAS_PER_SM) k_ngf_fused(FusedArgs a)
 
 // Batched fused pass: a persistent grid walks the tiles of all pairs.  Mode 0
 // evaluates at u; mode 1 at the trial point, for the pairs still searching.
+// searching[p]: whether pair p is evaluated, for the gather, whose own launch
+// takes the line-search decisions that change the states.
 template <bool HAS_DIR, typename IMG>
 __global__ void __launch_bounds__(BX * BY, CTAS_PER_SM) k_ngf_fused_batch(const PairLevel *__restrict__ pl,
                                                                 const int *__restrict__ tile_off, int npairs,
-                                                                int total)
+                                                                int total, int *__restrict__ searching)
 {
     extern __shared__ float sm[];
     for (int item = blockIdx.x; item < total; item += gridDim.x) {
         const int p = find_pair(tile_off, npairs, item);
         const PairLevel &P = pl[p];
-        if (HAS_DIR && !(P.st->active && P.st->ls_continue))
+        const bool skip = HAS_DIR && !(P.st->active && P.st->ls_continue);
+        if (item == __ldg(tile_off + p) && linear_tid() == 0)
+            searching[p] = !skip;
+        if (skip)
             continue;   // uniform over the CTA
         const FusedArgs &a = HAS_DIR ? P.fa_trial : P.fa_init;
         fused_tile<HAS_DIR, IMG, true, true>(a, item - __ldg(tile_off + p), sm);
@@ -670,8 +675,8 @@ cudaError_t launch_gather_grad_raw(const LevelGeom &g, const float *part, int nu
 // ---------------------------------------------------------------------------
 static bool g_batch_attr_set[64] = {};
 
-cudaError_t launch_fused_batch(const PairLevel *pl, const int *tile_off, int npairs, int total, int mode, bool bf16,
-                               int grid, int device, cudaStream_t s)
+cudaError_t launch_fused_batch(const PairLevel *pl, const int *tile_off, int npairs, int total, int *searching,
+                               int mode, bool bf16, int grid, int device, cudaStream_t s)
 {
     const int dev = device >= 0 && device < 64 ? device : 0;
     if (!g_batch_attr_set[dev]) {
@@ -691,28 +696,44 @@ cudaError_t launch_fused_batch(const PairLevel *pl, const int *tile_off, int npa
     if (bf16) {
         constexpr size_t SB = smem_bytes<__nv_bfloat16, true, true>();
         if (mode)
-            k_ngf_fused_batch<true, __nv_bfloat16><<<grid, blk, SB, s>>>(pl, tile_off, npairs, total);
+            k_ngf_fused_batch<true, __nv_bfloat16><<<grid, blk, SB, s>>>(pl, tile_off, npairs, total, searching);
         else
-            k_ngf_fused_batch<false, __nv_bfloat16><<<grid, blk, SB, s>>>(pl, tile_off, npairs, total);
+            k_ngf_fused_batch<false, __nv_bfloat16><<<grid, blk, SB, s>>>(pl, tile_off, npairs, total, searching);
     } else {
         constexpr size_t SB = smem_bytes<float, true, true>();
         if (mode)
-            k_ngf_fused_batch<true, float><<<grid, blk, SB, s>>>(pl, tile_off, npairs, total);
+            k_ngf_fused_batch<true, float><<<grid, blk, SB, s>>>(pl, tile_off, npairs, total, searching);
         else
-            k_ngf_fused_batch<false, float><<<grid, blk, SB, s>>>(pl, tile_off, npairs, total);
+            k_ngf_fused_batch<false, float><<<grid, blk, SB, s>>>(pl, tile_off, npairs, total, searching);
     }
     return cudaGetLastError();
 }
 
 namespace {
 
+// The rest of a batched evaluation in one launch.  Block p first reduces J, D
+// and S of pair p, which reads only the fused pass's block partials, and in
+// mode 1 takes the pair's line-search decision; the other blocks gather
+// meanwhile.  As launches of their own the reductions and the decisions were 3
+// of 6 launches of a line-search round: six pairs of 48^3 to 96^3, 2 levels,
+// 2559 -> 2384 us a batch.
 __global__ void __launch_bounds__(GATHER_NODES) k_gather_batch(const PairLevel *__restrict__ pl, const int *__restrict__ off,
-                                                      int npairs, int total, int mode)
+                                                      int npairs, int total, const int *__restrict__ searching, int mode)
 {
+    for (int p = blockIdx.x; p < npairs; p += gridDim.x) {
+        const PairLevel &P = pl[p];
+        if (!searching[p])
+            continue;   // uniform over the block
+        finalize_body(P.fa_init.partials, P.nD, P.pS, P.nS, P.hbar_half, P.alpha, P.hy_half, mode ? P.scal_t : P.scal);
+        __syncthreads();
+        if (mode == 1)
+            lb_control_body(LB_ARMIJO, P.st, nullptr, nullptr, 0, P.scal_t, 0ULL, 0ULL, 0ULL);
+        __syncthreads();
+    }
     for (int item = blockIdx.x; item < total; item += gridDim.x) {
         const int p = find_pair(off, npairs, item);
         const PairLevel &P = pl[p];
-        if (mode == 1 && !(P.st->active && P.st->ls_continue))
+        if (!searching[p])
             continue;
         const int lin = item - __ldg(off + p);
         const FusedArgs &a = P.fa_init;
@@ -723,10 +744,10 @@ __global__ void __launch_bounds__(GATHER_NODES) k_gather_batch(const PairLevel *
 
 }  // namespace
 
-cudaError_t launch_gather_batch(const PairLevel *pl, const int *off, int npairs, int total, int mode, int grid,
-                                cudaStream_t s)
+cudaError_t launch_gather_batch(const PairLevel *pl, const int *off, int npairs, int total, const int *searching,
+                                int mode, int grid, cudaStream_t s)
 {
-    k_gather_batch<<<grid, GATHER_NODES, 0, s>>>(pl, off, npairs, total, mode);
+    k_gather_batch<<<grid, GATHER_NODES, 0, s>>>(pl, off, npairs, total, searching, mode);
     return cudaGetLastError();
 }
 
