@@ -78,6 +78,7 @@ struct Level {
     int *tcnt[3] = {nullptr, nullptr, nullptr};
     float *tw[3] = {nullptr, nullptr, nullptr};
     int tmaxw[3] = {0, 0, 0};
+    int reach[3] = {0, 0, 0};   // most voxels in the two intervals of a node
     // prolongation from level + 1 onto this level's nodes
     int *qk0[3] = {nullptr, nullptr, nullptr};
     float *qw1[3] = {nullptr, nullptr, nullptr};

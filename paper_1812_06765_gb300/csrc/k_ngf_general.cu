@@ -47,7 +47,7 @@ constexpr int GSLOT_N = 3;                        // node planes: K and K + 1 in
 constexpr int GCOPY = (2 * GTP + NT - 1) / NT;
 constexpr int GCOMB = (GTP + NT - 1) / NT;
 constexpr int RROWS = OY;                         // rows of a completed node plane's columns
-constexpr int TAPS = 5;                           // voxels a node reaches per dimension below 2.5 voxels per interval
+constexpr int TAPS = 5;                           // voxels of a node's two intervals, below 2.5 voxels per interval
 static_assert(GNX == BX, "the x sums take one node column per thread of a row");
 
 // shared layout (floats)
@@ -86,9 +86,10 @@ struct GenArgs {
     double *partials;       // D block partials, one per tile
 };
 
-// One output tile (launch-order id, see tile_seg_col).  FEW: no node reaches
-// more than TAPS voxels along x or y, and the x and y sums take exactly TAPS
-// with weights from shared memory (zero where the node reaches fewer): no
+// One output tile (launch-order id, see tile_seg_col).  FEW: no node has
+// more than TAPS voxels in its two intervals along x or y (one that lies on the
+// node before it counts too, with its weight of 0), and the x and y sums take
+// exactly TAPS with weights from shared memory (zero where there are fewer): no
 // loop counters or tests, about half the instructions of the general sums.
 template <bool HAS_DIR, bool FEW>
 __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, float *sm)
@@ -663,7 +664,7 @@ cudaError_t launch_ngf_general(reg_ctx *c, int level, const float *ub, const flo
     *n_partials = a.ntx * a.nty * a.nseg;
     const dim3 blk(BX, BY, 1);
     const Level &L = c->L[level];
-    if (L.tmaxw[0] <= TAPS && L.tmaxw[1] <= TAPS)
+    if (L.reach[0] <= TAPS && L.reach[1] <= TAPS)
         dir ? k_ngf_general<true, true><<<*n_partials, blk, GSmem::BYTES, s>>>(a)
             : k_ngf_general<false, true><<<*n_partials, blk, GSmem::BYTES, s>>>(a);
     else

@@ -91,6 +91,7 @@ struct AxisTables {
     std::vector<int> k0, first, cnt;
     std::vector<float> w1, tw;   // tw[k * maxw + j]: weight of voxel first[k] + j for node k
     int maxw = 1;
+    int reach = 0;   // most voxels in the two intervals of a node (one on a node plane, of weight 0, included)
 };
 
 AxisTables axis_tables(int m, double h, double H, int n)
@@ -123,6 +124,13 @@ AxisTables axis_tables(int m, double h, double H, int n)
     for (int k = 0; k < n; k++) {
         a.cnt[k] = (int)ws[k].size();
         if (a.cnt[k] > a.maxw) a.maxw = a.cnt[k];
+    }
+    std::vector<int> in(n, 0);   // voxels per interval
+    for (int i = 0; i < m; i++)
+        in[a.k0[i]]++;
+    for (int k = 0; k < n; k++) {
+        const int r = (k > 0 ? in[k - 1] : 0) + in[k];
+        if (r > a.reach) a.reach = r;
     }
     a.tw.assign((size_t)n * a.maxw, 0.f);
     for (int k = 0; k < n; k++)
@@ -163,6 +171,7 @@ void carve_tables(Level &L, const AxisTables a[3], TableCarver &tc)
 {
     for (int d = 0; d < 3; d++) {
         L.tmaxw[d] = a[d].maxw;
+        L.reach[d] = a[d].reach;
         tc.put(L.pk0[d], a[d].k0);
         tc.put(L.pw1[d], a[d].w1);
         tc.put(L.tfirst[d], a[d].first);

@@ -19,6 +19,8 @@ FORMS = [
     ((90, 70, 64), (3, 3, 3)),            # intervals wider than a tile and longer than a segment
     ((60, 40, 32), (31, 11, 4)),          # ratios 2, 4 and 10.7
     ((61, 37, 43), (31, 5, 22)),          # 2.03, 9.25, 2.05
+    ((31, 21, 17), (13, 9, 7)),           # 5 weights a node, but 6 voxels in its intervals (one on a node)
+    ((41, 11, 25), (17, 5, 11)),          # the same, and exactly 2.5
 ]
 
 
