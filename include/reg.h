@@ -80,13 +80,14 @@ typedef struct reg_config {
     int start_level;      /* coarsest level solved; -1 = levels - 1 */
     int max_iter[REG_MAX_LEVELS];       /* accepted iterations per level (index = level) */
     int node_dims[REG_MAX_LEVELS][3];   /* deformation grid per level; 0 = m_d / 2 + 1 */
-    int eval_impl;        /* 0 fused objective pass; 1 multi-pass (intermediates in HBM,
+    int eval_impl;        /* 0 fused objective pass (grids of 2 or more voxels per node interval;
+                             denser node grids multi-pass); 1 multi-pass (intermediates in HBM,
                              P^T by the gather of Eq. 3); A/B baselines of P^T: 2 multi-pass
                              with an atomic scatter (summation order not fixed), 3 multi-pass
                              with an 8-colour scatter on ratio-2 levels (gather elsewhere) */
     int use_graph;        /* 1: each pyramid level runs as one CUDA graph launch */
     int image_dtype;      /* 0: FP32 images; 1: the fused pass reads BF16 copies of R and T
-                             (arithmetic stays FP32; levels without the fused pass use FP32) */
+                             (arithmetic stays FP32; levels of another ratio than 2 use FP32) */
     int autotune;         /* 1: reg_set_images times the z splits of the fused pass that a
                              load model ranks best on each level and keeps the fastest (cached
                              per geometry for the process; the first call of a geometry
@@ -120,7 +121,7 @@ typedef struct reg_stats {
     double level_seconds[REG_MAX_LEVELS]; /* device time of each level, its prolongation included
                                              (CUDA events on the handle's stream) */
     int tiling[REG_MAX_LEVELS];       /* fused-pass tiling per level: reg_register, the z segment
-                                         length (0: multi-pass level); reg_register_batch, the
+                                         length (0: ratio not 2); reg_register_batch, the
                                          rule the batch used (0 each pair's own tiling, -1 the
                                          throughput rule, T > 0 one segment length T) */
 } reg_stats;
@@ -163,8 +164,8 @@ int reg_level_info(reg_handle h, int level, int img_dims[3], int node_dims[3],
 /* Tiling of the fused objective pass on a level (no counterpart in the paper,
  * which uses separate kernels): *tz = the longest z segment (output planes per
  * CTA, chosen by the autotuner, cfg.fused_split, cfg.fused_tz or the load
- * model), *tiles = CTAs per evaluation.  Both 0 on levels the multi-pass
- * kernels serve.  Any output pointer may be NULL. */
+ * model), *tiles = CTAs per evaluation.  Both 0 on levels of another ratio
+ * than 2 (the general-ratio pass and the multi-pass kernels).  Any output pointer may be NULL. */
 int reg_level_tiling(reg_handle h, int level, int *tz, int *tiles);
 
 /* (No counterpart in the paper.)  The load model's z split of the fused pass
@@ -201,7 +202,7 @@ int reg_axis_tables(int m, double h, int n, int *k0, float *w1, int *first, int 
 /* (No counterpart in the paper.)  The z split of the fused pass on a level,
  * in the form of cfg.fused_split: split[5] = (l1, n1, l2, n2, lr), n1
  * segments of l1 planes, then n2 of l2, then lr planes (0: no remainder),
- * every tile column alike.  All 0 on levels the multi-pass kernels serve.
+ * every tile column alike.  All 0 on levels of another ratio than 2.
  * REG_ERR_STATE before reg_set_images. */
 int reg_level_split(reg_handle h, int level, int split[5]);
 
@@ -221,7 +222,7 @@ int reg_eval_objective_grad(reg_handle h, int level, const float *u_dev, float *
                             double *J, double *D, double *S);
 
 /* Device time (ms) of the NGF pass of the last reg_eval_objective_grad call on
- * this handle: the fused kernel (or the multi-pass NGF kernels), timed with
+ * this handle: the fused kernel of its ratio (or the multi-pass NGF kernels), timed with
  * CUDA events on the handle's stream around its launch; the curvature and
  * gradient-assembly kernels are not included.  Synchronises on that event.
  * REG_ERR_STATE before the first evaluation.  A profiling aid (the paper
