@@ -377,7 +377,9 @@ __device__ __forceinline__ void ld_corner_pair(const __nv_bfloat162 *p, float &a
 // The 8 corners of cell (cx, cy, cz) of the zero-bordered template (row pitch
 // MXP, MYP rows per plane, plane pitch SXYP).  Cells outside [-2, m] (padded
 // [0, m + 2]; CXM, CYM, CZM = m + 2) move to the far border, whose 8 corners
-// are zeros; so do the columns whose displacement is unusable (!ok).
+// are zeros; so do the columns whose displacement is unusable (!ok).  Their
+// value is 0 if their fractions are finite: zeros times a fraction that is not
+// are NaN (the general-ratio pass clears it; in the ratio-2 pass J is then NaN).
 template <typename ELEM>
 __device__ __forceinline__ void corners_padded(const ELEM *T, int cx, int cy, int cz, bool ok, unsigned CXM,
                                                unsigned CYM, unsigned CZM, int MXP, int MYP, size_t SXYP, float v[8])

@@ -272,6 +272,11 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
             // the displacement of every plane between them is below 1e6 voxels and finite
             ok0 = q0max.x < 1.0e6f && acc.x < 1.0e12f;
             ok1 = q0max.y < 1.0e6f && acc.y < 1.0e12f;
+            // a first node out of range: unusable on every plane of the interval
+            if (!(q0max.x < 1.0e6f))
+                Bl[0].x = Dd[0].x = NAN;
+            if (!(q0max.y < 1.0e6f))
+                Bl[0].y = Dd[0].y = NAN;
             if (!first) {   // plane K - 1's slot
                 issue_plane(K + 2);
                 pend = K + 2;
@@ -289,11 +294,27 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
             ix[0][c] = __float_as_int(fm.x);
             ix[1][c] = __float_as_int(fm.y);
         }
+        // An interval whose ends are not both in range (never in a registration that converges):
+        // sample_coord's test of the plane itself.  An unusable sample has the value and the
+        // gradient 0: its corners are zeros, and its fractions, which may not be finite, 0 too.
+        bool use0 = ok0, use1 = ok1;
+        if (!(ok0 && ok1)) {
+            use0 = use1 = true;
+#pragma unroll
+            for (int c = 0; c < 3; c++) {
+                const float2 q = mul2(lerp2(Bl[c], Dd[c], WZ), bc2(g.ih[c]));
+                use0 = use0 && fabsf(q.x) < 1.0e6f;   // false for NaN
+                use1 = use1 && fabsf(q.y) < 1.0e6f;
+            }
+#pragma unroll
+            for (int c = 0; c < 3; c++)
+                fr[c] = make_float2(use0 ? fr[c].x : 0.f, use1 ? fr[c].y : 0.f);
+        }
 #pragma unroll
         for (int k = 0; k < 2; k++) {
             float v[8];
             corners_padded(static_cast<const TemplateElem<float>::type *>(a.T), ix[k][0] + cb[k][0],
-                           ix[k][1] + cb[k][1], ix[k][2] + cb[k][2] + z1, k ? ok1 : ok0, CXM, CYM, CZM, MXP, MYP, SXYP,
+                           ix[k][1] + cb[k][1], ix[k][2] + cb[k][2] + z1, k ? use1 : use0, CXM, CYM, CZM, MXP, MYP, SXYP,
                            v);
 #pragma unroll
             for (int j = 0; j < 8; j++) {
