@@ -180,14 +180,17 @@ __device__ __forceinline__ float rcp_approx(float x)
 // and c' = a . bh + tau rh, the cosine is c = c' / sqrt(na2) and
 //   psi = 1 - c^2 = (|a x bh|^2 + |rh a - tau bh|^2) / na2   (no cancellation),
 //   v = d psi / d a = -2 (c' / na2) bh + 2 (c' / na2)^2 a,
-// so one reciprocal per lane serves both.
+// so one reciprocal per lane serves both.  TAU_FMA: tau^2 enters without being
+// rounded to FP32 itself (the rounding moves D by up to its own 6e-8: by -3.7e-8
+// at tau = 0.1, which the multi-pass kernels do not have).
+template <bool TAU_FMA>
 __device__ __forceinline__ float2 ngf_residual_rn2(const float2 a[3], const float2 bh[3], float2 rh, float tau,
                                                    float2 v[3])
 {
     const float2 TAU = bc2(tau), NTAU = bc2(-tau);
     const float2 aa = fma2(a[2], a[2], fma2(a[1], a[1], mul2(a[0], a[0])));
     const float2 ab = fma2(a[2], bh[2], fma2(a[1], bh[1], mul2(a[0], bh[0])));
-    const float2 na2 = add2(aa, bc2(tau * tau));
+    const float2 na2 = TAU_FMA ? fma2(TAU, TAU, aa) : add2(aa, bc2(tau * tau));
     const float2 cx = sub2(mul2(a[1], bh[2]), mul2(a[2], bh[1]));
     const float2 cy = sub2(mul2(a[2], bh[0]), mul2(a[0], bh[2]));
     const float2 cz = sub2(mul2(a[0], bh[1]), mul2(a[1], bh[0]));
@@ -398,6 +401,7 @@ __device__ __forceinline__ void corners_padded(const ELEM *T, int cx, int cy, in
 // R's normalized gradient field bn0, bn1 of the pair: (bx, bx'), (by, by') |
 // (bz, bz'), (rh, rh').  The x neighbours come from the threads beside it;
 // dyp, dym are the row steps (0 where the neighbour row is missing).
+template <bool TAU_FMA>
 __device__ __forceinline__ float2 ngf_pair_rn(const float *T0, const float *Tp, const float *Tm, int dyp, int dym,
                                               const float4 &bn0, const float4 &bn1, float2 HX, float2 HY, float2 HZ,
                                               float tau, float2 v[3])
@@ -410,7 +414,7 @@ __device__ __forceinline__ float2 ngf_pair_rn(const float *T0, const float *Tp, 
     const float2 av[3] = {mul2(make_float2(t0.y - tl, tr - t0.x), HX), mul2(sub2(typ, tym), HY),
                           mul2(sub2(tzp, tzm), HZ)};
     const float2 bh[3] = {make_float2(bn0.x, bn0.y), make_float2(bn0.z, bn0.w), make_float2(bn1.x, bn1.y)};
-    return ngf_residual_rn2(av, bh, make_float2(bn1.z, bn1.w), tau, v);
+    return ngf_residual_rn2<TAU_FMA>(av, bh, make_float2(bn1.z, bn1.w), tau, v);
 }
 
 // Phase C: the adjoint of the central differences at a pair of columns from
@@ -741,8 +745,8 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &a, int tile_id, floa
                 // rows 0 and BY - 1, whose v is never read, run the same code
                 const float *Tr = sm + SL::T + sp;
                 float2 v[3];
-                const float2 psi = ngf_pair_rn(Tr + (zB & 3) * PLANE, Tr + ((zB + 1) & 3) * PLANE,
-                                               Tr + ((zB - 1) & 3) * PLANE, dyp, dym, bn0, bn1, HX, HY, HZ, a.tau, v);
+                const float2 psi = ngf_pair_rn<false>(Tr + (zB & 3) * PLANE, Tr + ((zB + 1) & 3) * PLANE,
+                                                      Tr + ((zB - 1) & 3) * PLANE, dyp, dym, bn0, bn1, HX, HY, HZ, a.tau, v);
                 if (FULL || (zB >= z0 && zB < zend))
                     psi_sum.add(mul2(psi, MO));
                 float *vq = sm + SL::V + (zB & 3) * 3 * PLANE + sp;

@@ -418,8 +418,8 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
         if (FULL || (zB >= z0 - 1 && zB <= zend)) {
             const float *Tr = sm + SL::T + sp;
             float2 v[3];
-            const float2 psi = ngf_pair_rn(Tr + (zB & 3) * PLANE, Tr + ((zB + 1) & 3) * PLANE,
-                                           Tr + ((zB - 1) & 3) * PLANE, dyp, dym, bn0, bn1, HX, HY, HZ, a.tau, v);
+            const float2 psi = ngf_pair_rn<true>(Tr + (zB & 3) * PLANE, Tr + ((zB + 1) & 3) * PLANE,
+                                                 Tr + ((zB - 1) & 3) * PLANE, dyp, dym, bn0, bn1, HX, HY, HZ, a.tau, v);
             if (FULL || (zB >= z0 && zB < zend))
                 psi_sum.add(mul2(psi, MO));
             float *vq = sm + SL::V + (zB & 3) * 3 * PLANE + sp;
