@@ -64,7 +64,9 @@ struct GSmem {
     static constexpr int KY = KX + CW;
     static constexpr int FX = KY + BY;                   // first output column of each interval (int) [GNX + 2]
     static constexpr int FY = FX + GNX + 2;              // first output row [GNY + 2]
-    static constexpr int TWX = FY + GNY + 2;             // P^T weights of each node column [GNX][TAPS]
+    static constexpr int BX0 = FY + GNY + 2;             // first output column with a weight on each node column (int) [GNX]
+    static constexpr int BY0 = BX0 + GNX;                // first output row [GNY]
+    static constexpr int TWX = BY0 + GNY;                // P^T weights of each node column [GNX][TAPS]
     static constexpr int TWY = TWX + GNX * TAPS;         // and node row [GNY][TAPS]
     static constexpr int FLOATS = TWY + GNY * TAPS;
     static constexpr size_t BYTES = sizeof(float) * FLOATS;
@@ -121,6 +123,14 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
     const bool rowC = ty >= 2 && ty < BY - 2;
     const bool outxy = rowC && tx >= 1 && tx < BX - 1;
     const float2 MO = bc2(outxy ? 1.f : 0.f);     // psi is zero off the interior
+    // T~ counts where an interior voxel's central differences read it: on the interior and beside it,
+    // not on the image's edges or outside.  Bits 0, 1: of the pair's columns on the interior planes,
+    // 2, 3: on the first and the last plane.
+    // border coordinates of the pair's columns in x and y (4: outside).  T~ counts where an interior
+    // voxel's central differences read it: on the interior and beside it, at most one border
+    // coordinate with that of z; not on the image's edges or outside.
+    auto cls = [](int i, int m) { return i < 0 || i >= m ? 4 : i == 0 || i == m - 1 ? 1 : 0; };
+    const int c0 = cls(xa, mx) + cls(y, my), c1 = cls(xa + 1, mx) + cls(y, my);
     const int dyp = ty < BY - 1 ? CW : 0, dym = ty > 0 ? CW : 0;
     const int nz = g.n[2];
     const size_t node_plane = (size_t)g.n[0] * g.n[1];
@@ -128,6 +138,7 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
     // tables of the tile's columns and rows (positions outside the image take the border's)
     int *kxs = reinterpret_cast<int *>(sm + SL::KX), *kys = reinterpret_cast<int *>(sm + SL::KY);
     int *fx = reinterpret_cast<int *>(sm + SL::FX), *fy = reinterpret_cast<int *>(sm + SL::FY);
+    int *bx = reinterpret_cast<int *>(sm + SL::BX0), *by = reinterpret_cast<int *>(sm + SL::BY0);
     if (tid < CW) {
         const int i = min(max(x0 - 2 + tid, 0), mx - 1);
         kxs[tid] = __ldg(g.pk0[0] + i);
@@ -142,17 +153,29 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
     const int ocx = min(OX, mx - x0), ocy = min(OY, my - y0);  // output columns and rows in the image
     const int kox = kxs[2], koy = kys[2];                      // first node of the output columns
     const int nxl = kxs[1 + ocx] - kox + 2, nyl = kys[1 + ocy] - koy + 2;   // nodes they reach
-    // f[j + 1]: the first output column (row) in an interval >= j, for j = -1 .. GNX
+    // f[j + 1]: the first output column (row) in an interval >= j, for j = -1 .. GNX.  b[j]: that of the
+    // interval before node j, less one that lies on the node before (weight 0: a value there that is
+    // not finite must not reach node j)
     if (tid < GNX + 2) {
-        int f = 2;
-        for (int i = 2; i < 2 + ocx; i++)
-            f += kxs[i] - kox < tid - 1;
+        int f = 2, b = 2;
+        for (int i = 2; i < 2 + ocx; i++) {
+            const int k = kxs[i] - kox - (tid - 1);
+            f += k < 0;
+            b += k < 0 || (k == 0 && sm[SL::WX + i] == 0.f);
+        }
         fx[tid] = f;
+        if (tid < GNX)
+            bx[tid] = b;
     } else if (tid >= 64 && tid < 64 + GNY + 2) {
-        int f = 2;
-        for (int i = 2; i < 2 + ocy; i++)
-            f += kys[i] - koy < tid - 65;
+        int f = 2, b = 2;
+        for (int i = 2; i < 2 + ocy; i++) {
+            const int k = kys[i] - koy - (tid - 65);
+            f += k < 0;
+            b += k < 0 || (k == 0 && sm[SL::WY + i] == 0.f);
+        }
         fy[tid - 64] = f;
+        if (tid - 64 < GNY)
+            by[tid - 64] = b;
     }
     // the pair's node intervals: the second column lies in the first's or the next one
     const int lkx = kxs[2 * tx] - kx0, lky = kys[ty] - ky0;
@@ -335,17 +358,18 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
             const float *w = sm + SL::TWX + tx * TAPS, *r = src + (ty - 2) * CW + e0;
             float s0 = 0.f, s1 = 0.f, s2 = 0.f;
 #pragma unroll
-            for (int i = 0; i < TAPS; i++) {
-                s0 = fmaf(w[i], r[i], s0);
-                s1 = fmaf(w[i], r[RROWS * CW + i], s1);
-                s2 = fmaf(w[i], r[2 * RROWS * CW + i], s2);
-            }
+            for (int i = 0; i < TAPS; i++)
+                if (w[i] != 0.f) {   // predicated: a value that is not finite reaches no node without a weight on it
+                    s0 = fmaf(w[i], r[i], s0);
+                    s1 = fmaf(w[i], r[RROWS * CW + i], s1);
+                    s2 = fmaf(w[i], r[2 * RROWS * CW + i], s2);
+                }
             float *d = dst + (ty - 2) * GNX + tx;
             d[0] = s0;
             d[RROWS * GNX] = s1;
             d[2 * RROWS * GNX] = s2;
         } else if (!FEW && rowC && tx < nxl) {
-            const int e0 = fx[tx], e1 = fx[tx + 1], e2 = fx[tx + 2];
+            const int e0 = bx[tx], e1 = fx[tx + 1], e2 = fx[tx + 2];
             const float *r = src + (ty - 2) * CW;
             float s0 = 0.f, s1 = 0.f, s2 = 0.f;
             for (int i = e0; i < e2; i++) {
@@ -374,10 +398,11 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
                 float s = 0.f;
 #pragma unroll
                 for (int i = 0; i < TAPS; i++)
-                    s = fmaf(w[i], r[i * GNX], s);
+                    if (w[i] != 0.f)
+                        s = fmaf(w[i], r[i * GNX], s);
                 part_tile[(size_t)K * GNE + e] = s;
             } else if (!FEW && e < GNE && jy < nyl && jx < nxl) {
-                const int e0 = fy[jy], e1 = fy[jy + 1], e2 = fy[jy + 2];
+                const int e0 = by[jy], e1 = fy[jy + 1], e2 = fy[jy + 2];
                 const float *r = src + c * (RROWS * GNX) + jx;
                 float s = 0.f;
                 for (int i = e0; i < e2; i++) {
@@ -405,6 +430,11 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
         if (FULL || zA <= zend + 1) {
             float2 val, gx, gy, gz;
             interp_pair(pc, fr, val, gx, gy, gz);
+            // T~ where it does not count is 0: R's field is 0 off the interior, and so are psi and v, but
+            // not beside a T~ that is not finite.  (Selecting psi and v instead: 181 x 217 x 181 4 us
+            // and 256 x 256 x 112 on 65 x 65 x 29 nodes 3 us more an evaluation.)
+            const int lim = zA >= 1 && zA <= mz - 2 ? 1 : zA == 0 || zA == mz - 1 ? 0 : -1;
+            val = make_float2(c0 <= lim ? val.x : 0.f, c1 <= lim ? val.y : 0.f);
             sts2(sm + SL::T + (zA & 3) * PLANE + sp, val);
             float *gq = sm + SL::G + gs * 3 * PLANE + sp;
             sts2(gq, gx);
@@ -419,7 +449,7 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
             const float *Tr = sm + SL::T + sp;
             float2 v[3];
             const float2 psi = ngf_pair_rn<true>(Tr + (zB & 3) * PLANE, Tr + ((zB + 1) & 3) * PLANE,
-                                                 Tr + ((zB - 1) & 3) * PLANE, dyp, dym, bn0, bn1, HX, HY, HZ, a.tau, v);
+                                           Tr + ((zB - 1) & 3) * PLANE, dyp, dym, bn0, bn1, HX, HY, HZ, a.tau, v);
             if (FULL || (zB >= z0 && zB < zend))
                 psi_sum.add(mul2(psi, MO));
             float *vq = sm + SL::V + (zB & 3) * 3 * PLANE + sp;
@@ -476,7 +506,8 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
                 for (int c = 0; c < 3; c++) {
                     const float2 dT = lds2(gq + c * PLANE);
                     lo[c] = fma2(gl, dT, lo[c]);
-                    hi[c] = fma2(gh, dT, hi[c]);
+                    if (w != 0.f)   // uniform; a plane on a node plane has no weight on the next one
+                        hi[c] = fma2(gh, dT, hi[c]);
                 }
             }
         }

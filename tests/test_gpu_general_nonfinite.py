@@ -51,3 +51,16 @@ def test_unusable_displacements_are_outside_the_image(dims, nodes, value):
         u = random_field(nodes, 53, 1.0).astype(np.float32)
         u[comp, kz, ky, kx] = value
         assert_same(*both(dims, nodes, R, T, u))
+
+
+# T~ is not finite at voxels of an edge of the image, which no interior voxel's central difference
+# reads (u = 0: a cell reaches from a voxel to the next ones, so the edges at 0 in two dimensions)
+@pytest.mark.parametrize("value", [np.inf, np.nan])
+@pytest.mark.parametrize("dims,nodes", FORMS)
+def test_template_not_finite_off_the_interior(dims, nodes, value):
+    R, T = random_image(dims, 54), random_image(dims, 55)
+    mx, my, mz = dims
+    for z, y, x in [(0, 0, mx // 2), (0, my // 2, 0), (mz // 2, 0, 0), (0, 0, 0)]:
+        Tn = T.copy()
+        Tn[z, y, x] = value
+        assert_same(*both(dims, nodes, R, Tn, np.zeros((3,) + nodes[::-1], np.float32)))
