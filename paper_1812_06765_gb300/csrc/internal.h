@@ -74,6 +74,7 @@ struct Level {
     float4 *Rn = nullptr;
     int *pk0[3] = {nullptr, nullptr, nullptr};
     float *pw1[3] = {nullptr, nullptr, nullptr};
+    float *pw0[3] = {nullptr, nullptr, nullptr};   // weight of node k0 (general-ratio pass)
     int *tfirst[3] = {nullptr, nullptr, nullptr};
     int *tcnt[3] = {nullptr, nullptr, nullptr};
     float *tw[3] = {nullptr, nullptr, nullptr};

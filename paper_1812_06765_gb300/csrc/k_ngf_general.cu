@@ -60,7 +60,9 @@ struct GSmem {
     static constexpr int N = RX + 3 * RROWS * GNX;       // node planes [GSLOT_N][2][GTP]
     static constexpr int WX = N + GSLOT_N * 2 * GTP;     // weight of node k0 + 1, per column [CW]
     static constexpr int WY = WX + CW;                   // per row [BY]
-    static constexpr int KX = WY + BY;                   // k0 of the columns and rows (int)
+    static constexpr int WX0 = WY + BY;                  // weight of node k0 in P^T, per column [CW]
+    static constexpr int WY0 = WX0 + CW;                 // per row [BY]
+    static constexpr int KX = WY0 + BY;                  // k0 of the columns and rows (int)
     static constexpr int KY = KX + CW;
     static constexpr int FX = KY + BY;                   // first output column of each interval (int) [GNX + 2]
     static constexpr int FY = FX + GNX + 2;              // first output row [GNY + 2]
@@ -80,6 +82,7 @@ struct GenArgs {
     const float4 *Rn;       // R's normalized gradient field (row length rounded up to even)
     const float *ub, *dir;
     const double *t_dev;
+    const float *pw0[3];    // P^T: weight of a voxel on its node k0, per dimension
     float tau;
     FusedSplit split;       // z segments
     int nseg;               // their count
@@ -143,10 +146,12 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
         const int i = min(max(x0 - 2 + tid, 0), mx - 1);
         kxs[tid] = __ldg(g.pk0[0] + i);
         sm[SL::WX + tid] = __ldg(g.pw1[0] + i);
+        sm[SL::WX0 + tid] = __ldg(a.pw0[0] + i);
     } else if (tid >= 64 && tid < 64 + BY) {
         const int i = min(max(y0 - 2 + tid - 64, 0), my - 1);
         kys[tid - 64] = __ldg(g.pk0[1] + i);
         sm[SL::WY + tid - 64] = __ldg(g.pw1[1] + i);
+        sm[SL::WY0 + tid - 64] = __ldg(a.pw0[1] + i);
     }
     __syncthreads();
     const int kx0 = kxs[0], ky0 = kys[0];                      // first node of the node tile
@@ -247,7 +252,7 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
     int kq = __ldg(g.pk0[2] + zclamp(z0 - 2));
     float wq = __ldg(g.pw1[2] + zclamp(z0 - 2));
     int kc = __ldg(g.pk0[2] + z0);
-    float wc = __ldg(g.pw1[2] + z0);
+    float wc = __ldg(g.pw1[2] + z0), wc0 = __ldg(a.pw0[2] + z0);
     int Kc = kc;                   // node interval of phase C's sums
     int kx_pend = -1, ky_pend = -1;   // node planes whose x sums, y sums are due
 
@@ -373,8 +378,7 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
             const float *r = src + (ty - 2) * CW;
             float s0 = 0.f, s1 = 0.f, s2 = 0.f;
             for (int i = e0; i < e2; i++) {
-                const float w1 = sm[SL::WX + i];
-                const float w = i < e1 ? w1 : 1.f - w1;
+                const float w = sm[(i < e1 ? SL::WX : SL::WX0) + i];
                 s0 = fmaf(w, r[i], s0);
                 s1 = fmaf(w, r[RROWS * CW + i], s1);
                 s2 = fmaf(w, r[2 * RROWS * CW + i], s2);
@@ -406,8 +410,7 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
                 const float *r = src + c * (RROWS * GNX) + jx;
                 float s = 0.f;
                 for (int i = e0; i < e2; i++) {
-                    const float w1 = sm[SL::WY + i];
-                    s = fmaf(i < e1 ? w1 : 1.f - w1, r[(i - 2) * GNX], s);
+                    s = fmaf(sm[(i < e1 ? SL::WY : SL::WY0) + i], r[(i - 2) * GNX], s);
                 }
                 part_tile[(size_t)K * GNE + e] = s;
             }
@@ -477,11 +480,12 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
         // ---- C: r on plane zA - 4, summed along z into the interval's node planes
         const int zC = zA - 4;
         if (FULL || (zC >= z0 && zC < zend)) {
-            const float w = wc;
+            const float w = wc, w0 = wc0;
             const int K = kc;
             const int z2 = zclamp(zC + 1);
             kc = __ldg(g.pk0[2] + z2);
             wc = __ldg(g.pw1[2] + z2);
+            wc0 = __ldg(a.pw0[2] + z2);
             if (K != Kc) {   // the interval's lower plane is complete (uniform over the CTA)
                 store_plane(sm + SL::RZ, lo);
 #pragma unroll
@@ -501,7 +505,7 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
                 const float2 gj = adjoint_pair(V0, Vz + ((zC - 1) & 3) * 3 * PLANE, Vz + ((zC + 1) & 3) * 3 * PLANE, vx,
                                                vl, vr, HX, HY, HZ);
                 const float *gq = sm + SL::G + (gs == GSLOTS - 1 ? 0 : gs + 1) * 3 * PLANE + sp;
-                const float2 gh = mul2(gj, bc2(w)), gl = mul2(gj, bc2(1.f - w));
+                const float2 gh = mul2(gj, bc2(w)), gl = mul2(gj, bc2(w0));
 #pragma unroll
                 for (int c = 0; c < 3; c++) {
                     const float2 dT = lds2(gq + c * PLANE);
@@ -534,8 +538,8 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
         const int e = isx ? tid : tid - GNX * TAPS, j = e / TAPS;
         const int *f = (isx ? fx : fy) + j;
         const int i = e - j * TAPS + min(f[0], isx ? CW - TAPS : 2 + RROWS - TAPS);
-        const float w1 = sm[(isx ? SL::WX : SL::WY) + i];
-        sm[(isx ? SL::TWX : SL::TWY) + e] = i < f[0] || i >= f[2] ? 0.f : i < f[1] ? w1 : 1.f - w1;
+        sm[(isx ? SL::TWX : SL::TWY) + e] =
+            i < f[0] || i >= f[2] ? 0.f : sm[i < f[1] ? (isx ? SL::WX : SL::WY) + i : (isx ? SL::WX0 : SL::WY0) + i];
     }
     a_issue(z0 - 2, true);
     __syncthreads();
@@ -666,6 +670,8 @@ GenArgs general_args(const reg_ctx *c, int level, const float *ub, const float *
     a.ub = ub;
     a.dir = dir;
     a.t_dev = t_dev;
+    for (int d = 0; d < 3; d++)
+        a.pw0[d] = L.pw0[d];
     a.tau = (float)c->cfg.tau;
     a.split = L.gen_split;
     a.nseg = L.gen_split.count();

@@ -90,6 +90,7 @@ int validate_config(const reg_config *cfg, std::string &msg)
 struct AxisTables {
     std::vector<int> k0, first, cnt;
     std::vector<float> w1, tw;   // tw[k * maxw + j]: weight of voxel first[k] + j for node k
+    std::vector<float> w0;       // weight of node k0, rounded from FP64 as tw (1 - w1 is only within 3e-8 of it)
     int maxw = 1;
     int reach = 0;   // most voxels in the two intervals of a node (one on a node plane, of weight 0, included)
 };
@@ -99,6 +100,7 @@ AxisTables axis_tables(int m, double h, double H, int n)
     AxisTables a;
     a.k0.resize(m);
     a.w1.resize(m);
+    a.w0.resize(m);
     std::vector<double> t(m);
     for (int i = 0; i < m; i++) {
         t[i] = (i + 0.5) * h / H;
@@ -107,6 +109,7 @@ AxisTables axis_tables(int m, double h, double H, int n)
         if (k < 0) k = 0;
         a.k0[i] = k;
         a.w1[i] = (float)(t[i] - k);
+        a.w0[i] = (float)(1.0 - (t[i] - k));
     }
     a.first.assign(n, 0);
     a.cnt.assign(n, 0);
@@ -174,6 +177,7 @@ void carve_tables(Level &L, const AxisTables a[3], TableCarver &tc)
         L.reach[d] = a[d].reach;
         tc.put(L.pk0[d], a[d].k0);
         tc.put(L.pw1[d], a[d].w1);
+        tc.put(L.pw0[d], a[d].w0);
         tc.put(L.tfirst[d], a[d].first);
         tc.put(L.tcnt[d], a[d].cnt);
         tc.put(L.tw[d], a[d].tw);

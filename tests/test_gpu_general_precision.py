@@ -29,3 +29,37 @@ def test_d_has_no_bias(orc, tau):
         err.append((D - Do) / Do)
         r.close()
     assert abs(np.mean(err)) <= 1.5e-8, err
+
+
+@pytest.mark.parametrize("dims,nodes", [((361, 21, 19), None), ((361, 24, 20), (91, 7, 6)), ((25, 23, 721), None),
+                                        ((21, 361, 18), (9, 145, 7))])
+def test_small_weights_of_the_adjoint(dims, nodes):
+    """P^T's weight on the node before a voxel just below a node: a single bright template voxel, u = 0,
+    so that the voxels that the gradient sees share one index along the long axis, and the gradient at
+    the two nodes around it has exactly the ratio of the two weights.  1 - (FP32 weight of the other
+    node) is off by up to 3e-8 of weights of 1 / m; each side here is a dozen FP32 roundings: 2e-6."""
+    import paper_1812_06765_gb300 as reg
+    from paper_1812_06765_gb300 import _lib
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    nodes = nodes or tuple(m // 2 + 1 for m in dims)
+    axis = int(np.argmax(dims))
+    k0, w1 = _lib.reg_axis_tables(dims[axis], 1.0, nodes[axis])[:2]
+    t = (np.arange(dims[axis]) + 0.5) * (nodes[axis] - 1) / dims[axis]
+    low = 1.0 - (t - k0)                                        # the lower node's weight in 64 bits
+    loss = np.abs((np.float32(1) - np.asarray(w1, np.float32)).astype(np.float64) - low) / low
+    loss[:8] = loss[-8:] = 0
+    i = int(np.argmax(loss))
+    assert loss[i] > 4e-6                                       # the voxel where rounding the other weight shows most
+    p = [m // 2 for m in dims]
+    p[axis] = i
+    R, T = random_image(dims, 90), np.zeros(dims[::-1], np.float32)
+    T[p[2], p[1], p[0]] = 1.0
+    r = reg.Registration(reg.make_config(levels=1, tau=0.06, alpha=1.0, node_dims=[nodes])).set_images(R, T, (1.0,) * 3)
+    g = r.eval(torch.zeros((3,) + nodes[::-1], device="cuda"))[3].cpu().numpy().astype(np.float64)
+    r.close()
+    g = np.moveaxis(g[1 if axis == 0 else 0], 2 - axis, 0)      # a component across the axis, the axis first
+    lo, hi = g[k0[i]], g[k0[i] + 1]
+    j = np.unravel_index(np.argmax(np.abs(hi)), hi.shape)
+    assert hi[j] != 0
+    assert abs(lo[j] / hi[j] - low[i] / (1.0 - low[i])) <= 2e-6 * low[i] / (1.0 - low[i])
