@@ -124,6 +124,35 @@ __device__ __forceinline__ DFloat df_add(DFloat a, DFloat b)
 __device__ __forceinline__ DFloat df_add(DFloat a, float b) { return df_add(a, DFloat{b, 0.f}); }
 __device__ __forceinline__ double df_to_double(DFloat a) { return (double)a.hi + (double)a.lo; }
 
+// Block sum of one double-float per thread as FP64 in thread 0 (other threads:
+// 0), for blocks whose totals hold so many terms that FP32 totals would round
+// more than the terms' own sums do.  The order is that of block_sum_to_f64.
+// sm holds >= nwarps pairs.
+__device__ __forceinline__ DFloat warp_sum(DFloat v)
+{
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1)
+        v = df_add(v, DFloat{__shfl_xor_sync(0xffffffffu, v.hi, o), __shfl_xor_sync(0xffffffffu, v.lo, o)});
+    return v;
+}
+__device__ __forceinline__ double block_sum_to_f64(DFloat v, DFloat *sm)
+{
+    const int tid = linear_tid();
+    const int nw = (nthreads() + 31) / 32;
+    v = warp_sum(v);
+    if ((tid & 31) == 0)
+        sm[tid >> 5] = v;
+    __syncthreads();
+    double s = 0.0;
+    if (tid < 32) {
+        const DFloat x = warp_sum(tid < nw ? sm[tid] : DFloat{0.f, 0.f});
+        if (tid == 0)
+            s = df_to_double(x);
+    }
+    __syncthreads();
+    return s;
+}
+
 // Ordered FP64 sum (is_max: max) of count values x[i0], x[i0 + step], ...,
 // starting from s.  The loads go out 8 at a time so that their L2 round trips
 // overlap; the additions keep the index order, so the result is the plain

@@ -573,8 +573,10 @@ __device__ __forceinline__ void general_tile(const GenArgs &a, int tile_id, floa
     __syncthreads();
     y_sums(sm + SL::V, Kc);
     y_sums(sm + SL::V + 3 * PLANE, Kc + 1);
-    const float2 ps = psi_sum.s;
-    const double ssum = block_sum_to_f64(ps.x + ps.y, reinterpret_cast<double *>(sm + SL::RZ));
+    // a tile's total holds tens of thousands of terms (the multi-pass kernels round one of 256 to FP32)
+    const float2 ps = psi_sum.s, pe = psi_sum.c;
+    const double ssum = block_sum_to_f64(df_add(DFloat{ps.x, -pe.x}, DFloat{ps.y, -pe.y}),
+                                         reinterpret_cast<DFloat *>(sm + SL::RZ));
     if (tid == 0)
         a.partials[tile_id] = ssum;
 }

@@ -63,3 +63,20 @@ def test_small_weights_of_the_adjoint(dims, nodes):
     j = np.unravel_index(np.argmax(np.abs(hi)), hi.shape)
     assert hi[j] != 0
     assert abs(lo[j] / hi[j] - low[i] / (1.0 - low[i])) <= 2e-6 * low[i] / (1.0 - low[i])
+
+
+def test_tile_totals_of_d_are_not_rounded():
+    """Ramps across each other: psi is the same FP32 number at every interior voxel, so D / (hbar / 2) over
+    their count is that number again, up to the FP64 and double-float sums (2^-46, 1e-10 allows for 10^3
+    of them); a tile total rounded to FP32 would leave up to 6e-8."""
+    import paper_1812_06765_gb300 as reg
+    if not torch.cuda.is_available():
+        pytest.skip("no CUDA device")
+    for dims in [(61, 57, 49), (85, 43, 131), (29, 13, 21)]:
+        z, y, x = np.meshgrid(*[np.arange(m) for m in dims[::-1]], indexing="ij")
+        R, T = (x / 64.0).astype(np.float32), (y / 128.0).astype(np.float32)
+        r = reg.Registration(reg.make_config(levels=1, tau=0.07, rho=0.03, alpha=1.0)).set_images(R, T, (1.0,) * 3)
+        D = r.eval(torch.zeros((3,) + tuple(m // 2 + 1 for m in dims[::-1]), device="cuda"))[1]
+        r.close()
+        psi = D / (0.5 * np.prod([m - 2 for m in dims]))
+        assert abs(psi - float(np.float32(psi))) <= 1e-10 * psi, (dims, psi)
