@@ -721,7 +721,8 @@ __device__ __forceinline__ void pair_coefficients(LbfgsState &S, int count, doub
     set_compact_warp(&S);
 }
 
-template <int C>
+// SPREAD: the elements are spread over the grid instead of taken by chunks of PD_CHUNK
+template <int C, bool SPREAD>
 __global__ void __launch_bounds__(VT) k_lb_pair_dots(long long n, const float *__restrict__ S,
                                                      const float *__restrict__ Y, const float *__restrict__ g,
                                                      float *__restrict__ partials, unsigned *__restrict__ cnt,
@@ -732,11 +733,13 @@ __global__ void __launch_bounds__(VT) k_lb_pair_dots(long long n, const float *_
 #pragma unroll
     for (int d = 0; d < ND; d++)
         v[d] = 0.f;
-    for (long long e0 = blockIdx.x * (long long)PD_CHUNK; e0 < n; e0 += (long long)gridDim.x * PD_CHUNK) {
+    const long long step = SPREAD ? (long long)gridDim.x * VT : VT;
+    for (long long e0 = blockIdx.x * (long long)(SPREAD ? VT : PD_CHUNK) + threadIdx.x; e0 < n;
+         e0 += (long long)gridDim.x * PD_CHUNK) {
         float a[PD_U][2 * C + 1];
 #pragma unroll
         for (int k = 0; k < PD_U; k++) {
-            const long long e = e0 + k * VT + threadIdx.x;
+            const long long e = e0 + k * step;
             const bool in = e < n;
             a[k][2 * C] = in ? __ldg(g + e) : 0.f;
 #pragma unroll
@@ -842,11 +845,18 @@ template <int C>
 cudaError_t launch_pair_direction(reg_ctx *c, long long n, const float *S, const float *Y, const float *g, float *p,
                                   double Hmin, cudaStream_t s)
 {
-    // 2 blocks per SM: enough loads in flight, few partials for the last block
+    // Up to one chunk per SM the elements are spread over the grid, one to PD_U per thread, so that
+    // the threads' FP32 sums stay as short as that allows: chunks of 4 per thread on few blocks took
+    // the error of a direction of 3 x 7^3 unknowns from 7.0e-8 to 9.7e-8.  From there on chunks, on 2
+    // blocks per SM: enough loads in flight, few partials for the last block, and sums half as long as
+    // with a block per SM (3 x 129^3, 5 pairs: 126 us, spread 153 us; the errors agree to 1 %).
     const long long chunks = (n + PD_CHUNK - 1) / PD_CHUNK;
-    const int nb = (int)std::min<long long>(chunks, 2LL * c->num_sms);
+    const bool spread = chunks <= c->num_sms;
+    const int nb = (int)(spread ? std::min<long long>((n + VT - 1) / VT, c->num_sms)
+                                : std::min<long long>(chunks, 2LL * c->num_sms));
     const int nc = (int)std::min<long long>(chunks, 8LL * c->num_sms);
-    k_lb_pair_dots<C><<<nb, VT, 0, s>>>(n, S, Y, g, c->lb.partials, c->lb.cnt + c->lb.cnt_len, c->lb.st, Hmin);
+    const auto dots = spread ? k_lb_pair_dots<C, true> : k_lb_pair_dots<C, false>;
+    dots<<<nb, VT, 0, s>>>(n, S, Y, g, c->lb.partials, c->lb.cnt + c->lb.cnt_len, c->lb.st, Hmin);
     k_lb_pair_combine<C><<<nc, VT, 0, s>>>(n, c->lb.st, g, S, Y, p);
     c->launches += 2;
     return cudaGetLastError();
