@@ -351,7 +351,9 @@ int allocate_buffers(reg_ctx *c)
     Carver at;
     at.base = static_cast<char *>(c->arena);
     carve(at);
-    CK(cudaMemcpy(c->arena, table_host.data(), table_bytes, cudaMemcpyHostToDevice));
+    // in the order of the handle's stream, which the side stream follows: a copy on the default stream
+    // is ordered with neither, and may still be under way when the call returns
+    CK(cudaMemcpyAsync(c->arena, table_host.data(), table_bytes, cudaMemcpyHostToDevice, c->stream));
     CK(cudaMemsetAsync(at.base + zero_begin, 0, zero_end - zero_begin, c->stream));
     // page-locked, readable and writable from the device: the state's mirror and an evaluation's [J, D, S]
     void *host = nullptr;
