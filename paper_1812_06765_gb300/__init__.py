@@ -80,7 +80,6 @@ class Registration:
         self.stream = stream if stream is not None else torch.cuda.current_stream()
         self.h = _lib.reg_create(self.cfg, self.stream.cuda_stream)
         self.dims = None
-        self._shapes = {}   # node_shape per level, until the next images
 
     # -- images -------------------------------------------------------------
     def set_images(self, R, T, spacing):
@@ -101,7 +100,6 @@ class Registration:
             raise ValueError("R and T must be 3D arrays of equal shape")
         mz, my, mx = R.shape
         self.dims = (mx, my, mz)
-        self._shapes = {}
         _lib.reg_set_images(self.h, pr, pt, self.dims, spacing, dev)
         self._keep = (R, T)  # device copies are taken on the handle's stream
         return self
@@ -119,11 +117,8 @@ class Registration:
         return _lib.reg_level_split(self.h, level)
 
     def node_shape(self, level=0):
-        shape = self._shapes.get(level)
-        if shape is None:
-            n = self.level_info(level)["nodes"]
-            shape = self._shapes[level] = (3, n[2], n[1], n[0])
-        return shape
+        n = _lib.reg_level_nodes(self.h, level)
+        return (3, n[2], n[1], n[0])
 
     def level_image(self, level, which="R"):
         m = self.level_info(level)["dims"]

@@ -159,6 +159,16 @@ def reg_level_info(h, level):
     return tuple(m), tuple(n), tuple(sp), tuple(H)
 
 
+_INT3 = ctypes.c_int * 3
+
+
+def reg_level_nodes(h, level):
+    """The node counts of reg_level_info alone (1 us instead of 4: every call on a displacement asks for them)."""
+    n = _INT3()
+    check(h, lib().reg_level_info(h, int(level), None, n, None, None))
+    return n[0], n[1], n[2]
+
+
 def reg_level_tiling(h, level):
     tz, tiles = ctypes.c_int(), ctypes.c_int()
     check(h, lib().reg_level_tiling(h, int(level), ctypes.byref(tz), ctypes.byref(tiles)))
