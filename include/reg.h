@@ -86,8 +86,14 @@ typedef struct reg_config {
                              with an atomic scatter (summation order not fixed), 3 multi-pass
                              with an 8-colour scatter on ratio-2 levels (gather elsewhere) */
     int use_graph;        /* 1: each pyramid level runs as one CUDA graph launch */
-    int image_dtype;      /* 0: FP32 images; 1: the fused pass reads BF16 copies of R and T
-                             (arithmetic stays FP32; levels of another ratio than 2 use FP32) */
+    int image_dtype;      /* 0: FP32 images; 1: the fused pass takes R and T rounded to BF16
+                             (arithmetic stays FP32; levels of another ratio than 2 use FP32).
+                             Device memory of the images, with either: 12 bytes per voxel (R, T
+                             and the pass's copy of T), and 16 more for R's normalized gradient
+                             field on levels of more than 40 000 nodes and levels of another
+                             ratio.  With fused_tz = -1 ratio-2 levels keep no field: 12 bytes,
+                             for evaluations that take longer (256^3 349 -> 426 us, with BF16
+                             356 -> 472 us; 128^3, few of that form's tiles, 83 -> 192 us) */
     int autotune;         /* 1: reg_set_images times the z splits of the fused pass that a
                              load model ranks best on each level and keeps the fastest (cached
                              per geometry for the process; the first call of a geometry

@@ -27,7 +27,8 @@ def make_config(levels=1, tau=0.01, rho=None, alpha=10.0, mem=5, max_iter=50, c1
                 node_dims=None, eval_impl=None, use_graph=None, image_dtype=None, autotune=None, fused_tz=None,
                 fused_split=None):
     """A reg_config; max_iter is one value for every level or a per-level list (index 0 = finest).
-    image_dtype: "f32" (default) or "bf16" (the fused pass reads BF16 copies of the images).
+    image_dtype: "f32" (default) or "bf16" (the fused pass takes the images rounded to BF16, in as much
+    device memory: 28 bytes a voxel, or 12 with fused_tz=-1, for either).
     autotune: time the fused pass's z splits per level (default on); fused_tz: force equal segments
     of that length; fused_split: force (l1, n1, l2, n2, lr) on levels of that depth."""
     cfg = _lib.reg_config_default()

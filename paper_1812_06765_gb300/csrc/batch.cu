@@ -29,11 +29,11 @@ void fill_pair_level(reg_ctx *c, int level, PairLevel &P)
     FusedSplit split;
     int ntx, nty;
     fused_tiling(L, c->num_sms, &split, &ntx, &nty);
-    const bool bf16 = c->cfg.image_dtype == 1 && L.Tb && L.Rb;
+    const bool bf16 = c->cfg.image_dtype == 1 && L.Tb;
     FusedArgs a{};
     a.g = P.geom;
     a.T = bf16 ? static_cast<const void *>(L.Tb) : static_cast<const void *>(L.Tp);   // zero-bordered copies
-    a.R = bf16 ? static_cast<const void *>(L.Rb) : static_cast<const void *>(L.R);
+    a.R = L.R;
     a.Rn = L.Rn;
     a.ub = c->lb.u;
     a.dir = nullptr;

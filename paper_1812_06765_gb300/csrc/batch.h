@@ -7,8 +7,8 @@
 // Arguments of the fused objective pass over one pair (k_ngf_fused.cu).
 struct FusedArgs {
     LevelGeom g;
-    const void *T, *R;      // images, elements of the kernel's IMG type (float or bf16; a handle's T: TemplateElem)
-    const float4 *Rn;       // R's normalized gradient field (a handle's; else null)
+    const void *T, *R;      // images: T's elements of the kernel's IMG type (float or bf16; a handle's: TemplateElem), R's float
+    const float4 *Rn;       // R's normalized gradient field (of levels that read it; else null)
     const float *ub, *dir;
     const double *t_dev;
     float tau, rho;

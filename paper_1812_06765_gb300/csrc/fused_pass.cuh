@@ -60,11 +60,13 @@ struct Smem {
     static_assert((R | V | G | RED | N | PLANE) % 2 == 0, "float2 rows need even offsets");
 };
 // The single-pair pass over a handle's images (zero-bordered T) reads R's
-// normalized gradient field, BF16 images too (of R rounded to BF16: 16 bytes a
-// voxel instead of an R ring and its gradient in every evaluation).  R itself is read by the caller's own buffers (no field exists), and
-// by the passes that form the curvature too (the batched pass, whose persistent
-// kernel has no registers left for the field's prefetch and whose pairs would
-// stream 16 bytes per voxel each, and the single-pair form of its arithmetic).
+// normalized gradient field (of R rounded to BF16 for BF16 images): 16 bytes a
+// voxel instead of an R ring and its gradient in every evaluation.  R itself
+// is read from the caller's own buffers (no field exists), and by the passes
+// that form the curvature too (the batched pass, whose persistent kernel has no
+// registers left for the field's prefetch and whose pairs would stream 16 bytes
+// per voxel each, and the single-pair form of its arithmetic): a level whose
+// single-pair pass is one of those keeps no field (field_read).
 template <typename IMG, bool PAD, bool CURV>
 __host__ __device__ constexpr bool reads_rn()
 {
@@ -318,11 +320,14 @@ __device__ __forceinline__ void column_pair_plane(const float *nodes, int K, int
 // image element loads: FP32, or BF16 widened to FP32 (all arithmetic is FP32)
 __device__ __forceinline__ float ldimg(const float *p) { return __ldg(p); }
 __device__ __forceinline__ float ldimg(const __nv_bfloat16 *p) { return __bfloat162float(__ldg(p)); }
-// two adjacent elements starting at an even index (8- or 4-byte aligned)
+// two adjacent elements starting at an even index
 __device__ __forceinline__ float2 ldimg2(const float *p) { return __ldg(reinterpret_cast<const float2 *>(p)); }
-__device__ __forceinline__ float2 ldimg2(const __nv_bfloat16 *p)
+// two of R's values as images of type IMG hold them.  R stays FP32 in memory and BF16 images round it
+// where it is used: a BF16 copy beside it would be memory that no pass needs.
+template <typename IMG>
+__device__ __forceinline__ float2 as_image(float2 v)
 {
-    return __bfloat1622float2(__ldg(reinterpret_cast<const __nv_bfloat162 *>(p)));
+    return std::is_same<IMG, float>::value ? v : __bfloat1622float2(__float22bfloat162_rn(v));
 }
 
 template <typename IMG>
@@ -510,7 +515,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &a, int tile_id, floa
     const size_t node_plane = (size_t)g.n[0] * g.n[1];
     const IMG *Tim = static_cast<const IMG *>(a.T);   // the caller's template (not PAD)
     const auto *Tpad = static_cast<const typename TemplateElem<IMG>::type *>(a.T);
-    const IMG *Rcol = static_cast<const IMG *>(a.R) + (col_in ? xa + mx * y : 0);
+    const float *Rcol = static_cast<const float *>(a.R) + (col_in ? xa + mx * y : 0);
     // the pair's two 16-byte halves of R's normalized field (stored by column pair)
     const float4 *Rncol = RN ? a.Rn + (col_in ? xa + mx * y : 0) : nullptr;
     // padded template: row pitch, plane pitch and the largest cell index (padded coordinates)
@@ -727,7 +732,7 @@ __device__ __forceinline__ void fused_tile(const FusedArgs &a, int tile_id, floa
             const int slot = zA & 3;
             sts2(sm + SL::T + slot * PLANE + sp, val);
             if (!RN)
-                sts2(sm + SL::R + slot * PLANE + sp, rnext);
+                sts2(sm + SL::R + slot * PLANE + sp, as_image<IMG>(rnext));
             float *gq = sm + SL::G + gs * 3 * PLANE + sp;
             sts2(gq, gx);
             sts2(gq + PLANE, gy);

@@ -64,11 +64,10 @@ struct Level {
     long long nv, nn;
     float *R = nullptr, *T = nullptr;        // device images
     // read by the fused passes (general-ratio: FP32 always): T with a 2-voxel zero border on every side (dims m + 4), FP32
-    // (image_dtype 0) or BF16 x pairs (Tb, image_dtype 1, beside the BF16 copy Rb of R)
+    // (image_dtype 0) or BF16 x pairs (Tb, image_dtype 1; R is rounded where it is read)
     float *Tp = nullptr;
-    __nv_bfloat16 *Rb = nullptr;
     __nv_bfloat162 *Tb = nullptr;
-    // read by the fused passes beside Tp: R's normalized gradient field (b / ||b||_rho,
+    // read by the fused passes beside them (field_read): R's normalized gradient field (b / ||b||_rho,
     // rho / ||b||_rho) per voxel, b the central-difference gradient; zero off the interior;
     // rows of an odd length carry one more column of zeros
     float4 *Rn = nullptr;
@@ -170,13 +169,12 @@ inline int curv_planes(const int n[3])
 
 // launchers (return cudaError_t of the launch)
 cudaError_t launch_restrict(const float *src, const int m[3], float *dst, cudaStream_t s);
-cudaError_t launch_to_bf16(const float *src, __nv_bfloat16 *dst, long long n, cudaStream_t s);
 // the zero-bordered copy of a volume of dims m read by the fused pass (dims m + 4)
 long long padded_voxels(const int m[3]);
 cudaError_t launch_pad_template(const float *src, const int m[3], float *dst, cudaStream_t s);
 // BF16: element x holds (T[x], T[x + 1])
 cudaError_t launch_pad_template(const float *src, const int m[3], __nv_bfloat162 *dst, cudaStream_t s);
-// of R, or of R rounded to BF16 (its copy L.Rb)
+// of R, or with BF16 images of R rounded to BF16
 cudaError_t launch_ref_normal_field(const Level &L, double rho, cudaStream_t s);
 cudaError_t launch_prolong(const Level &coarse, const Level &fine, const float *uc, float *uf, cudaStream_t s);
 
@@ -301,6 +299,13 @@ inline bool small_level(const reg_ctx *c, int level) { return c->L[level].nn <= 
 inline bool fused_curv_in_pass(const reg_ctx *c, int level)
 {
     return c->cfg.fused_tz == -1 || small_level(c, level);
+}
+
+// Whether a pass of the level reads R's normalized gradient field, 16 of the 28 bytes a voxel that a
+// handle's images take with it (R, T, the pass's copy of T and the field).
+inline bool field_read(const reg_ctx *c, int level)
+{
+    return use_general(c, level) || (use_fused(c, level) && !fused_curv_in_pass(c, level));
 }
 
 // P^T of the multi-pass path: 0 node-centric gather (Eq. 3; eval_impl 0 and 1),

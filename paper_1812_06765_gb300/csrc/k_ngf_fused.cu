@@ -393,9 +393,9 @@ FusedArgs fused_args(const reg_ctx *c, int level, const float *ub, const float *
     const Level &L = c->L[level];
     FusedArgs a;
     a.g = L.geom();
-    const bool bf16 = c->cfg.image_dtype == 1 && L.Tb && L.Rb;
+    const bool bf16 = c->cfg.image_dtype == 1 && L.Tb;
     a.T = bf16 ? static_cast<const void *>(L.Tb) : static_cast<const void *>(L.Tp);   // zero-bordered copies
-    a.R = bf16 ? L.Rb : static_cast<const void *>(L.R);
+    a.R = L.R;
     a.Rn = L.Rn;
     a.ub = ub;
     a.dir = dir;
@@ -418,9 +418,9 @@ cudaError_t launch_ngf_fused(reg_ctx *c, int level, const float *ub, const float
 {
     (void)grad;
     const Level &L = c->L[level];
-    const bool bf16 = c->cfg.image_dtype == 1 && L.Tb && L.Rb;
-    if (!L.Rn)
-        return cudaErrorInvalidValue;   // handles keep R's normalized field beside the padded T
+    const bool bf16 = c->cfg.image_dtype == 1 && L.Tb;
+    if (field_read(c, level) && !L.Rn)
+        return cudaErrorInvalidValue;   // such levels keep R's normalized field beside the padded T
     int ntiles = 0;
     const FusedArgs a = fused_args(c, level, ub, dir, t_dev, partials, &ntiles);
     dim3 blk(BX, BY, 1), grd(ntiles, 1, 1);
@@ -530,7 +530,7 @@ std::map<std::array<int, 6>, FusedSplit> g_tune;
 cudaError_t fused_autotune(reg_ctx *c, int level, const float *u_zero, cudaStream_t s)
 {
     Level &L = c->L[level];
-    const bool bf16 = c->cfg.image_dtype == 1 && L.Tb && L.Rb;
+    const bool bf16 = c->cfg.image_dtype == 1 && L.Tb;
     const std::array<int, 6> key{L.m[0], L.m[1], L.m[2], c->num_sms, bf16 ? 1 : 0, c->device};
     {
         std::lock_guard<std::mutex> lk(g_tune_mu);

@@ -66,21 +66,6 @@ __global__ void k_prolong(const float *__restrict__ uc, int cx, int cy, int cz, 
     }
 }
 
-// FP32 -> BF16 (round to nearest even) image copy, float4 reads.
-__global__ void __launch_bounds__(256) k_to_bf16(const float *__restrict__ src, __nv_bfloat16 *__restrict__ dst,
-                                                 long long n)
-{
-    const long long n4 = n >> 2;
-    for (long long e = blockIdx.x * 256LL + threadIdx.x; e < n4; e += (long long)gridDim.x * 256) {
-        float4 v = reinterpret_cast<const float4 *>(src)[e];
-        __nv_bfloat162 a = __floats2bfloat162_rn(v.x, v.y), b = __floats2bfloat162_rn(v.z, v.w);
-        reinterpret_cast<__nv_bfloat162 *>(dst)[2 * e] = a;
-        reinterpret_cast<__nv_bfloat162 *>(dst)[2 * e + 1] = b;
-    }
-    if (blockIdx.x == 0 && threadIdx.x < (n & 3))
-        dst[4 * n4 + threadIdx.x] = __float2bfloat16_rn(src[4 * n4 + threadIdx.x]);
-}
-
 template <int V>
 struct VecOf;
 template <>
@@ -151,19 +136,21 @@ __global__ void __launch_bounds__(256) k_pad_template(const float *__restrict__ 
     }
 }
 
-__device__ __forceinline__ float ld_img(const float *p) { return __ldg(p); }
-__device__ __forceinline__ float ld_img(const __nv_bfloat16 *p) { return __bfloat162float(__ldg(p)); }
-// columns x (even) and x + 1; EVEN: even row length, one aligned load
-template <bool EVEN>
-__device__ __forceinline__ float2 ld_img_pair(const float *p)
+// R's values, with BF16 images rounded to BF16 (to nearest even)
+template <bool BF16>
+__device__ __forceinline__ float ld_ref(const float *p)
 {
-    return EVEN ? __ldg(reinterpret_cast<const float2 *>(p)) : make_float2(__ldg(p), __ldg(p + 1));
+    const float v = __ldg(p);
+    return BF16 ? __bfloat162float(__float2bfloat16_rn(v)) : v;
 }
-template <bool EVEN>
-__device__ __forceinline__ float2 ld_img_pair(const __nv_bfloat16 *p)
+// columns x (even) and x + 1; EVEN: even row length, one aligned load
+template <bool BF16, bool EVEN>
+__device__ __forceinline__ float2 ld_ref_pair(const float *p)
 {
-    return EVEN ? __bfloat1622float2(__ldg(reinterpret_cast<const __nv_bfloat162 *>(p)))
-                : make_float2(ld_img(p), ld_img(p + 1));
+    if (!EVEN)
+        return make_float2(ld_ref<BF16>(p), ld_ref<BF16>(p + 1));
+    const float2 v = __ldg(reinterpret_cast<const float2 *>(p));
+    return BF16 ? __bfloat1622float2(__float22bfloat162_rn(v)) : v;
 }
 
 // R's normalized gradient field for the fused pass (Eq. 2): R is fixed for the
@@ -192,8 +179,8 @@ __device__ __forceinline__ float quotient(float a, float b, float r)
     const float q = a * r;
     return fmaf(fmaf(-q, b, a), r, q);
 }
-template <typename TIN, bool EVEN>
-__global__ void __launch_bounds__(256) k_ref_normal_field(const TIN *__restrict__ R, int mx, int my, int mz, float hx,
+template <bool BF16, bool EVEN>
+__global__ void __launch_bounds__(256) k_ref_normal_field(const float *__restrict__ R, int mx, int my, int mz, float hx,
                                                           float hy, float hz, float rho, float4 *__restrict__ out, int planes)
 {
     const int x = 2 * (blockIdx.x * blockDim.x + threadIdx.x);
@@ -203,20 +190,20 @@ __global__ void __launch_bounds__(256) k_ref_normal_field(const TIN *__restrict_
     if (x >= mxe || y >= my)
         return;
     const size_t sy = (size_t)mx, sz = (size_t)mx * my;
-    const TIN *p = R + x + sy * y + sz * z0;
+    const float *p = R + x + sy * y + sz * z0;
     float4 *o = out + x + (size_t)mxe * (y + (size_t)my * z0);
     const bool iny = y >= 1 && y <= my - 2;
     const bool in0 = iny && x >= 1 && x <= mx - 2, in1 = iny && x + 1 <= mx - 2;
     // a pair holds an interior column: then both its columns and x - 1 or x + 2 are in the image
     const bool any = in0 || in1;
     const float2 zero = make_float2(0.f, 0.f);
-    float2 below = any && z0 > 0 ? ld_img_pair<EVEN>(p - sz) : zero, at = any ? ld_img_pair<EVEN>(p) : zero;
+    float2 below = any && z0 > 0 ? ld_ref_pair<BF16, EVEN>(p - sz) : zero, at = any ? ld_ref_pair<BF16, EVEN>(p) : zero;
     for (int z = z0; z < z1; z++, p += sz, o += (size_t)mxe * my) {
         float4 a = make_float4(0.f, 0.f, 0.f, 0.f), b = a;
-        const float2 above = any && z < mz - 1 ? ld_img_pair<EVEN>(p + sz) : zero;
+        const float2 above = any && z < mz - 1 ? ld_ref_pair<BF16, EVEN>(p + sz) : zero;
         if (any && z >= 1 && z <= mz - 2) {
-            const float2 up = ld_img_pair<EVEN>(p + sy), dn = ld_img_pair<EVEN>(p - sy);
-            const float l = in0 ? ld_img(p - 1) : 0.f, r = in1 ? ld_img(p + 2) : 0.f;
+            const float2 up = ld_ref_pair<BF16, EVEN>(p + sy), dn = ld_ref_pair<BF16, EVEN>(p - sy);
+            const float l = in0 ? ld_ref<BF16>(p - 1) : 0.f, r = in1 ? ld_ref<BF16>(p + 2) : 0.f;
             auto field = [&](float bx, float by, float bz, float &ox, float &oy, float &oz, float &orho) {
                 const float nb = sqrtf(fmaf(bz, bz, fmaf(by, by, bx * bx)) + rho * rho);
                 if (nb > 1e-30f && nb < 1e30f) {
@@ -261,8 +248,8 @@ cudaError_t launch_pad(const float *src, const int m[3], TOUT *dst, cudaStream_t
     return cudaGetLastError();
 }
 
-template <typename TIN>
-cudaError_t launch_field(const TIN *R, const Level &L, double rho, cudaStream_t s)
+template <bool BF16>
+cudaError_t launch_field(const Level &L, double rho, cudaStream_t s)
 {
     // the pass's difference factors: 0.5 * (float)(1 / h), as in grad T~
     const LevelGeom g = L.geom();
@@ -272,10 +259,10 @@ cudaError_t launch_field(const TIN *R, const Level &L, double rho, cudaStream_t 
     const int planes = L.nv >= MARCH_FROM ? FIELD_PLANES : 1;
     const dim3 grd((pairs + 31) / 32, (L.m[1] + 7) / 8, (L.m[2] + planes - 1) / planes);
     if (L.m[0] % 2 == 0)
-        k_ref_normal_field<TIN, true><<<grd, blk, 0, s>>>(R, L.m[0], L.m[1], L.m[2], hx, hy, hz, (float)rho, L.Rn,
+        k_ref_normal_field<BF16, true><<<grd, blk, 0, s>>>(L.R, L.m[0], L.m[1], L.m[2], hx, hy, hz, (float)rho, L.Rn,
                                                          planes);
     else
-        k_ref_normal_field<TIN, false><<<grd, blk, 0, s>>>(R, L.m[0], L.m[1], L.m[2], hx, hy, hz, (float)rho, L.Rn,
+        k_ref_normal_field<BF16, false><<<grd, blk, 0, s>>>(L.R, L.m[0], L.m[1], L.m[2], hx, hy, hz, (float)rho, L.Rn,
                                                          planes);
     return cudaGetLastError();
 }
@@ -296,16 +283,7 @@ cudaError_t launch_pad_template(const float *src, const int m[3], __nv_bfloat162
 
 cudaError_t launch_ref_normal_field(const Level &L, double rho, cudaStream_t s)
 {
-    return L.Rb ? launch_field(L.Rb, L, rho, s) : launch_field(L.R, L, rho, s);
-}
-
-cudaError_t launch_to_bf16(const float *src, __nv_bfloat16 *dst, long long n, cudaStream_t s)
-{
-    long long blocks = ((n >> 2) + 255) / 256;
-    if (blocks < 1) blocks = 1;
-    if (blocks > 4096) blocks = 4096;
-    k_to_bf16<<<(int)blocks, 256, 0, s>>>(src, dst, n);
-    return cudaGetLastError();
+    return L.Tb ? launch_field<true>(L, rho, s) : launch_field<false>(L, rho, s);
 }
 
 cudaError_t launch_restrict(const float *src, const int m[3], float *dst, cudaStream_t s)

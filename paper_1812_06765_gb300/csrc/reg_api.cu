@@ -313,15 +313,14 @@ int allocate_buffers(reg_ctx *c)
             Level &L = c->L[l];
             m.take(L.R, L.nv);
             m.take(L.T, L.nv);
-            // the fused passes read T through a zero-bordered copy (FP32, or BF16 beside a BF16 R)
+            // the fused passes read T through a zero-bordered copy (FP32, or pairs of BF16)
             if (use_fused(c, l) || use_general(c, l)) {
-                if (cfg.image_dtype == 1 && use_fused(c, l)) {
-                    m.take(L.Rb, L.nv);
+                if (cfg.image_dtype == 1 && use_fused(c, l))
                     m.take(L.Tb, padded_voxels(L.m));
-                } else {
+                else
                     m.take(L.Tp, padded_voxels(L.m));
-                }
-                m.take(L.Rn, rn_voxels(L.m));
+                if (field_read(c, l))
+                    m.take(L.Rn, rn_voxels(L.m));
             }
         }
         if (mp_vox > 0) {
@@ -513,10 +512,9 @@ int reg_set_images(reg_handle c, const float *R, const float *T, const int dims[
         c->launches += 2;
     }
     for (int l = 0; l < c->levels; l++) {
-        if (c->L[l].Rb) {
-            CK(launch_to_bf16(c->L[l].R, c->L[l].Rb, c->L[l].nv, c->stream));
+        if (c->L[l].Tb) {
             CK(launch_pad_template(c->L[l].T, c->L[l].m, c->L[l].Tb, c->side));
-            c->launches += 2;
+            c->launches += 1;
         }
         if (c->L[l].Tp) {
             CK(launch_pad_template(c->L[l].T, c->L[l].m, c->L[l].Tp, c->side));
