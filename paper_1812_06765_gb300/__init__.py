@@ -110,11 +110,11 @@ class Registration:
         return dict(dims=m, nodes=n, spacing=h, node_spacing=H)
 
     def level_tiling(self, level=0):
-        """(longest z segment, CTAs) of the fused pass on a level; (0, 0) for multi-pass levels."""
+        """(longest z segment, CTAs) of the fused pass on a level; (0, 0) where the ratio is not 2."""
         return _lib.reg_level_tiling(self.h, level)
 
     def level_split(self, level=0):
-        """(l1, n1, l2, n2, lr): the fused pass's z segments on a level; zeros for multi-pass levels."""
+        """(l1, n1, l2, n2, lr): the fused pass's z segments on a level; zeros where the ratio is not 2."""
         return _lib.reg_level_split(self.h, level)
 
     def node_shape(self, level=0):

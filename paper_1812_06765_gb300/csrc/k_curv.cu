@@ -5,7 +5,8 @@
 //   S   = hbar_y / 2 sum_c sum_k w_c^2
 //   grad_c J += alpha hbar_y L^T w_c     (the symmetric stencil gathered over
 //                                         the zero-extended w)
-// Both passes are node-parallel, one thread per node and all 3 components.
+// Both passes are node-parallel, all 3 components of a node in one thread (the
+// first takes up to 4 node planes per thread).
 #include "internal.h"
 #include "ngf_math.cuh"
 
@@ -138,7 +139,7 @@ cudaError_t launch_eval(reg_ctx *c, int level, const float *ub, const float *dir
     const bool fused = use_fused(c, level), general = use_general(c, level);
     const bool curv_in_pass = fused && fused_curv_in_pass(c, level);
     // The curvature Laplacian (node pass, HBM-light) runs on the side stream
-    // beside the NGF pass (issue-bound, one CTA per SM), in the tail of its last
+    // beside the NGF pass (issue-bound, two CTAs per SM that hold all its registers), in the tail of its last
     // wave: fork before, join before the gradient assembly.  Captured, the two
     // become parallel graph branches.  With the batched form's arithmetic the
     // fused pass forms it itself, with one S partial per tile.

@@ -110,8 +110,8 @@ __device__ __forceinline__ void vec_tail(const VecTail &t, const float *__restri
     lb_control_body(t.phase, t.st, nullptr, t.gpart, ng, t.scal, t.h_ls, t.h_iter, t.h_redo, preloaded);
 }
 
-// All vector passes read and write 16-byte vectors: u, g, gt and pdir are
-// separate allocations and the P / Y ring slots sit at a stride that is a
+// All vector passes read and write 16-byte vectors: u, g, gt and pdir start at
+// 256-byte boundaries and the P / Y ring slots sit at a stride that is a
 // multiple of 4 floats.  The n % 4 tail is done by the first threads of block 0.
 __device__ __forceinline__ float dot4(float4 a, float4 b) { return a.x * b.x + a.y * b.y + a.z * b.z + a.w * b.w; }
 __device__ __forceinline__ float max4(float4 a)
@@ -676,7 +676,9 @@ __global__ void k_batch_condition(const PairLevel *__restrict__ pl, int npairs, 
 // the loads are 4-byte ones, coalesced, PD_U per vector and thread in flight.
 // 3 x 65^3 unknowns, 5 pairs: one pass per dot, the sums and the solve in one
 // FP64 thread and FP64 coefficients per element took 166 + 1292 + 54 us, the
-// whole call 1481 us; now the call takes 49 us.
+// whole call 1481 us; now the call takes 42-48 us.  PD_U: with 2 elements in
+// flight 46 us of device time, with 4 43, with 8 46; 3 x 129^3: 151, 126 and
+// 136 us.
 constexpr int PD_U = 4;                     // elements per thread and chunk
 constexpr int PD_CHUNK = PD_U * VT;
 
@@ -849,7 +851,8 @@ cudaError_t launch_pair_direction(reg_ctx *c, long long n, const float *S, const
     // the threads' FP32 sums stay as short as that allows: chunks of 4 per thread on few blocks took
     // the error of a direction of 3 x 7^3 unknowns from 7.0e-8 to 9.7e-8.  From there on chunks, on 2
     // blocks per SM: enough loads in flight, few partials for the last block, and sums half as long as
-    // with a block per SM (3 x 129^3, 5 pairs: 126 us, spread 153 us; the errors agree to 1 %).
+    // with a block per SM (3 x 129^3, 5 pairs: 126 us, spread 153 us, 1 block per SM 133 us, 4 135 us;
+    // 3 x 65^3: 43, 46, 39 and 51 us).  The combination's grid: 2, 4 and 8 blocks per SM agree to 2 %.
     const long long chunks = (n + PD_CHUNK - 1) / PD_CHUNK;
     const bool spread = chunks <= c->num_sms;
     const int nb = (int)(spread ? std::min<long long>((n + VT - 1) / VT, c->num_sms)

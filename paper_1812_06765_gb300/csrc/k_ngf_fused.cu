@@ -714,9 +714,13 @@ namespace {
 // The rest of a batched evaluation in one launch.  Block p first reduces J, D
 // and S of pair p, which reads only the fused pass's block partials, and in
 // mode 1 takes the pair's line-search decision; the other blocks gather
-// meanwhile.  As launches of their own the reductions and the decisions were 3
-// of 6 launches of a line-search round: six pairs of 48^3 to 96^3, 2 levels,
-// 2559 -> 2384 us a batch.
+// meanwhile.  As launches of their own the reductions and the decisions were 2
+// of 5 launches of a line-search round (pass, gather, reduction, decision,
+// condition): six pairs of 48^3 to 96^3, 2 levels, 2559 -> 2384 us a batch.
+// They cost every block registers and shared memory (64 and 10.4 KB, 4 blocks
+// per SM instead of 5), which large batches do not show: 64 pairs of 96^3 to
+// 224^2 x 160, 3 levels of 60 iterations 723.8 -> 722.5 ms, 8 pairs of 256^3
+// with 10 iterations a level 85.1 -> 84.4 ms, 4 of 512 x 512 x 256 149.6 -> 147.5.
 __global__ void __launch_bounds__(GATHER_NODES) k_gather_batch(const PairLevel *__restrict__ pl, const int *__restrict__ off,
                                                       int npairs, int total, const int *__restrict__ searching, int mode)
 {

@@ -22,13 +22,19 @@
 //          instead of once per voxel plane.
 //
 // What bounds it: as the ratio-2 pass, issue, latency and L1 together (181 x
-// 217 x 181: 105 M warp instructions, issue active 0.50, L1 66 %, DRAM 11 %,
-// 190 us).  The four kernels of the multi-pass form (k_ngf_multipass.cu) it
+// 217 x 181: 114 M warp instructions, issue active 0.54, L1 67 %, DRAM 11 %,
+// 187 us).  The four kernels of the multi-pass form (k_ngf_multipass.cu) it
 // replaces moved about 100 bytes per voxel through HBM and gathered P^T with
 // scalar loads.  A whole evaluation, multi-pass -> this pass: 181 x 217 x 181
 // with 91 x 109 x 91 nodes 415 -> 257 us, 256 x 256 x 112 with 65 x 65 x 29
 // nodes 498 -> 233 us (equal z segments instead of the uneven split, and the
-// x and y sums with run-time windows: 282 and 241 us).
+// x and y sums with run-time windows: 282 and 241 us); with the curvature and
+// host side of the calls since, 237 and 220 us.
+//
+// Values that are not finite or out of range go as far as in the multi-pass
+// kernels: a sample without a usable displacement is outside the image, a
+// voxel reaches the nodes on which it has a weight, and the image's edges,
+// which no interior difference reads, do not reach D.
 #include "internal.h"
 #include "lbfgs_control.cuh"
 

@@ -170,10 +170,17 @@ __device__ __forceinline__ float2 ld_ref_pair(const float *p)
 // stride 8 took 47 us at 256 x 256 x 112, and with four separate divisions
 // (163 instructions a voxel) 42 us; now 29 us (86 instructions).
 constexpr int FIELD_PLANES = 4;
-constexpr long long MARCH_FROM = 1 << 20;   // voxels from which a thread takes several planes
+// Voxels from which a thread of the field and of the padded copy takes several
+// planes.  4 planes against 1, field + copy: 129 x 127 x 123 (2.0 M) 17.2
+// against 19.8 us, 161 x 159 x 151 27.1 against 35.0, 255 x 257 x 113 53
+// against 62, even rows within 2 us of each other; 97 x 95 x 91 and 96^3 (0.8 M)
+// within 1 us, where too few blocks would be left on smaller volumes.
+constexpr long long MARCH_FROM = 1 << 20;
 // a / b, correctly rounded, from r = 1 / b correctly rounded: one residual
 // correction of a r (Markstein's theorem, IBM J. Res. Dev. 34, 1990; b and r in
-// the normal range).  Several quotients of one divisor share r.
+// the normal range, and |a| from 2^-102 up or 0: the residual of a smaller a
+// underflows, and the last bit of a quotient may then differ).  Several
+// quotients of one divisor share r.
 __device__ __forceinline__ float quotient(float a, float b, float r)
 {
     const float q = a * r;
